@@ -7,7 +7,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libsso.so")
-SOURCES = ["elements.cu", "assembly.cu", "pcg.cu", "coarse.cu", "chain.cu", "spmv.cu", "spmv_noalloc.cu",
+SOURCES = ["elements.cu", "assembly.cu", "pcg.cu", "cluster.cu", "coarse.cu", "chain.cu", "spmv.cu", "spmv_noalloc.cu",
            "small.cu", "capi.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",

@@ -168,6 +168,8 @@ struct HostTopo {
   // the K blocks (i, j) with i in g and j in h, in block order
   int n_agg = 0;
   std::vector<int> agg_of, agg_ptr, agg_nodes, cg_ptr, cg_src;
+  // block positions of the tiles (one-cluster CG), exclusive prefix
+  std::vector<int> toff;
   // block (i, i+1) of every node or -1, and whether every block lies within
   // one of the diagonal (a chain)
   std::vector<int> chain_up;
@@ -230,6 +232,12 @@ struct sso_model {
   double penal = 1.0;
   // SSO_CHAIN: the pattern is block-tridiagonal; workspace of the factors
   // (allocated on first use), assembly count when they were formed
+  // one-cluster CG: whether the structure fits the engine, and per cluster
+  // size the largest share of a CTA
+  bool cluster_ok = false;
+  int cl_positions = 0;
+  ClusterShare cl_share[CL_SIZES] = {};
+  int* d_toff;
   bool is_chain = false;
   int* d_chain_up;        // [n_nodes] block (i, i+1) or -1
   double* d_chain_ws = nullptr;
@@ -304,9 +312,13 @@ struct sso_batch {
   std::vector<cudaEvent_t> part_ev;
   // the models' set-up jobs (one launch per set-up stage for the whole batch)
   SetupJob* d_jobs = nullptr;
-  // SSO_F32X2: the systems being solved (one CTA each)
+  // SSO_F32X2: the systems being solved (one CTA each); one-cluster CG: the
+  // systems by cluster size
   int* d_list = nullptr;
   std::vector<int> h_list;
+  // one-cluster CG: extra streams for the launches of further cluster sizes
+  cudaStream_t cl_stream[2 * CL_SIZES - 1] = {};
+  cudaEvent_t cl_fork = nullptr, cl_join[2 * CL_SIZES - 1] = {};
   SetupExtent extent;
   cudaEvent_t ev = nullptr;
   // kernel timing (sso_batch_set_profiling): events around every A and B
@@ -634,6 +646,9 @@ bool topology_consistent(const HostMesh& m, const HostTopo& T) {
 
 int n_chunks_of(const sso_model* M) { return (M->n_tiles + CHUNK - 1) / CHUNK; }
 
+// One-cluster CG: bytes of a model's packed K, in the element-block scratch.
+size_t cluster_pack_bytes(const sso_model* M) { return (size_t)M->cl_positions * CL_POS_BYTES; }
+
 // Lays out (base == nullptr: sizes only) every device array of a model.
 size_t layout_model(sso_model* M, void* base) {
   Carver c(base);
@@ -664,6 +679,7 @@ size_t layout_model(sso_model* M, void* base) {
   M->d_cg_ptr = c.take<int>(na * na + 1);
   M->d_cg_src = c.take<int>(M->n_blocks);
   M->d_chain_up = c.take<int>(n);
+  M->d_toff = c.take<int>((n + TILE - 1) / TILE + 1);
   // element blocks; after assembly also the Galerkin block products
   M->d_ke = c.take<double>((size_t)std::max(M->n_eb, M->n_blocks) * 36);
   M->d_fslot = c.take<double>(M->n_slots);
@@ -1030,6 +1046,175 @@ sso_status chain_run(sso_batch* B, const sso_options* o, bool adjoint,
 
 sso_status finish_run(sso_batch* B, const std::vector<char>& active, sso_stats* stats);
 
+// ---------------------------------------------------------------------------
+// One-cluster CG (cluster.cu) of a batch's systems.
+
+// One launch: `n` systems from list entry `first`, clusters of `size` CTAs.
+struct ClusterBin {
+  int first, n, size, threads, smem;
+  bool m_tm;  // the preconditioner in tensor memory
+};
+
+// What the device holds at once (cluster_limits).
+struct ClusterDevice {
+  int smem = 0, slots[CL_SIZES];
+};
+sso_status cluster_device(const ClusterDevice** out) {
+  static std::mutex mu;
+  static ClusterDevice d;
+  std::lock_guard<std::mutex> lock(mu);
+  if (!d.smem) {
+    ClusterDevice q;
+    CK(cluster_limits(&q.smem, q.slots));
+    d = q;
+  }
+  *out = &d;
+  return SSO_OK;
+}
+
+// Warps of a CTA: as few rounds of tiles per warp as the limit allows, evenly
+// filled.
+int cluster_warps(int own_tiles) {
+  const int most = CL_MAX_THREADS / 32, rounds = (own_tiles + most - 1) / most;
+  return std::max(2, (own_tiles + rounds - 1) / rounds);
+}
+
+// How a structure runs when n_sys run together: the cluster size (index; -1:
+// the two-kernel engine), and whether tensor memory holds the preconditioner.
+// The least estimated time of all n_sys: an iteration is the barriers,
+// reductions and vector updates (kClusterFixed clocks) plus, per round of
+// tiles, the products (kClusterRound) plus the part of K that comes from L2 at
+// 64 bytes a clock and SM; systems beyond the clusters resident at once run in
+// waves.  Measured (clocks of an iteration, estimate in brackets),
+// 64 x 64 shells: size 16 15,200 (14,500), size 9 22,100 (20,000); 64 33 x 33
+// shells, us a system-iteration: size 2 0.292, 3 0.311, 4 0.257, 6 0.294, 9
+// 0.53.  The systems in flight must fit L2 (kClusterL2 bytes of it) with the
+// part of K that is not resident: it would else come from HBM in every
+// iteration, where the two-kernel engine is as fast.
+constexpr size_t kClusterL2 = (size_t)100 << 20;
+constexpr double kClusterFixed = 9500.0, kClusterRound = 5000.0;
+struct ClusterChoice {
+  int size = -1;
+  bool m_tm = false;
+};
+ClusterChoice cluster_choice(const sso_model* M, int n_sys, int precond,
+                             const ClusterDevice& d) {
+  ClusterChoice best;
+  if (!M->cluster_ok) return best;
+  double best_t = HUGE_VAL;
+  for (int k = 0; k < CL_SIZES; ++k) {
+    const ClusterShare& sh = M->cl_share[k];
+    const int C = cl_size_of(k), slots = d.slots[k], warps = cluster_warps(sh.own_tiles);
+    if (slots < 1 || sh.window >= 65535 || (k > 0 && M->n_tiles < 2 * C)) continue;
+    // The preconditioner in shared memory, or in tensor memory (CTAs that use
+    // all of their shared memory anyway), whichever leaves less of K to L2; a
+    // position of K per warp in shared memory at least: the ring behind L2.
+    // (In tensor memory a 100 x 100 grid shell, two-level, fits at all: 33.2 ->
+    // 17.7 ms a solve; a 64 x 64 shell, two-level, 26.0 -> 25.7 ms.)
+    const size_t share = (size_t)CL_POS_BYTES * sh.positions;
+    size_t stream = SIZE_MAX;
+    bool m_tm = false;
+    for (int in_tm = 0; in_tm < (precond == SSO_JACOBI ? 1 : 2); ++in_tm) {
+      const size_t need = cluster_smem_bytes(sh, precond, in_tm);
+      const int pos = cluster_tm_positions(d.smem, sh.own_tiles, warps, in_tm);
+      if (pos < 0 || need + (size_t)CL_POS_BYTES * warps > (size_t)d.smem ||
+          (in_tm && need + share <= (size_t)d.smem))
+        continue;
+      const size_t resident = d.smem - need + (size_t)CL_POS_BYTES * warps * pos;
+      const size_t rest = share - std::min(share, resident);
+      if (rest < stream) {
+        stream = rest;
+        m_tm = in_tm;
+      }
+    }
+    if (stream == SIZE_MAX) continue;
+    if ((size_t)std::min(slots, n_sys) * C * stream > kClusterL2) continue;
+    const double rounds = (double)sh.own_tiles / warps;
+    const double t = kClusterFixed + kClusterRound * rounds + stream / 64.0;
+    const double waves = n_sys <= slots ? 1.0 : (double)n_sys / slots;
+    if (t * waves < best_t) {
+      best_t = t * waves;
+      best.size = k;
+      best.m_tm = m_tm;
+    }
+  }
+  return best;
+}
+
+// Sorts the active systems into launches by cluster size; *fits is false when
+// a system does not fit the engine (the batch then runs the two-kernel engine).
+template <class GetModel>
+sso_status plan_bins(int n_sys, const std::vector<char>& active, int precond, GetModel model,
+                     std::vector<int>& list, std::vector<ClusterBin>& bins, bool* fits) {
+  *fits = false;
+  list.clear();
+  bins.clear();
+  const ClusterDevice* dev = nullptr;
+  sso_status st = cluster_device(&dev);
+  if (st != SSO_OK) return st;
+  int n_act = 0;
+  for (int s = 0; s < n_sys; ++s) n_act += active[s] != 0;
+  std::vector<ClusterChoice> choice(n_sys);
+  for (int s = 0; s < n_sys; ++s) {
+    if (!active[s]) continue;
+    choice[s] = cluster_choice(model(s), n_act, precond, *dev);
+    if (choice[s].size < 0) return SSO_OK;
+  }
+  for (int k = CL_SIZES - 1; k >= 0; --k)
+    for (int m_tm = 0; m_tm < 2; ++m_tm) {
+      ClusterBin b{(int)list.size(), 0, cl_size_of(k), 0, 0, m_tm != 0};
+      for (int s = 0; s < n_sys; ++s) {
+        if (choice[s].size != k || choice[s].m_tm != b.m_tm) continue;
+        const ClusterShare& sh = model(s)->cl_share[k];
+        // all of a CTA's K resident where it fits, else whatever room is left
+        const size_t all = m_tm ? dev->smem
+                                : cluster_smem_bytes(sh, precond, false) +
+                                      (size_t)CL_POS_BYTES * (sh.positions + 2);
+        b.smem = std::max(b.smem, (int)std::min((size_t)dev->smem, all));
+        b.threads = std::max(b.threads, 32 * cluster_warps(sh.own_tiles));
+        list.push_back(s);
+        ++b.n;
+      }
+      if (b.n) bins.push_back(b);
+    }
+  *fits = !list.empty();
+  return SSO_OK;
+}
+
+// One round: up to max_steps CG steps of every system of the bins, each bin
+// on a stream of its own, joined back to B's stream.
+sso_status launch_bins(sso_batch* B, const std::vector<ClusterBin>& bins, const int* d_list,
+                       int precond, int max_steps) {
+  const int nb = (int)bins.size();
+  if (nb > 1) {
+    if (!B->cl_fork) CK(cudaEventCreateWithFlags(&B->cl_fork, cudaEventDisableTiming));
+    for (int k = 0; k < nb - 1; ++k) {
+      if (!B->cl_stream[k])
+        CK(cudaStreamCreateWithFlags(&B->cl_stream[k], cudaStreamNonBlocking));
+      if (!B->cl_join[k]) CK(cudaEventCreateWithFlags(&B->cl_join[k], cudaEventDisableTiming));
+    }
+    CK(cudaEventRecord(B->cl_fork, B->stream));
+  }
+  for (int k = 0; k < nb; ++k) {
+    const ClusterBin& b = bins[k];
+    cudaStream_t s = k == 0 ? B->stream : B->cl_stream[k - 1];
+    if (k > 0) CK(cudaStreamWaitEvent(s, B->cl_fork, 0));
+    CL(launch_cluster_cg(B->d_sys, d_list + b.first, b.n, b.size, b.threads, b.smem, precond,
+                         b.m_tm, B->d_n_active, max_steps, s),
+       1);
+    if (k > 0) {
+      CK(cudaEventRecord(B->cl_join[k - 1], s));
+      CK(cudaStreamWaitEvent(B->stream, B->cl_join[k - 1], 0));
+    }
+  }
+  return SSO_OK;
+}
+
+// CG steps of a system per launch: long enough that loading a system (some
+// microseconds) does not count, short enough that the host sees finished
+// systems and the wall-clock cap within a few milliseconds.
+constexpr int kClusterSteps = 1024;
+
 // defer: return after queuing the copy of the scalars, without waiting (the
 // caller synchronises the stream and calls finish_run).
 sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
@@ -1045,6 +1230,15 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
                        B->stream));
     for (int s = 0; s < B->n_sys; ++s) B->h_sys[s].tile0 = B->h_tile0[s];
     B->compacted = false;
+  }
+  // FP32 CG with one cluster per system where every system fits it; profiled
+  // runs time the two-kernel engine's launches
+  bool cluster = false;
+  std::vector<ClusterBin> bins;
+  if (o->precision == SSO_FP32_IR && !B->profiling) {
+    sso_status st = plan_bins(B->n_sys, active, o->precond,
+                              [B](int s) { return B->models[s]; }, B->h_list, bins, &cluster);
+    if (st != SSO_OK) return st;
   }
   int n_act = 0;
   for (int s = 0; s < B->n_sys; ++s) {
@@ -1100,6 +1294,30 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
     CL(launch_small_cg(B->d_sys, B->d_list, (int)B->h_list.size(), threads, max_nodes,
                        o->precond == SSO_TWO_LEVEL, B->stream),
        2);
+  } else if (n_act > 0 && cluster) {
+    CK(cudaMemcpyAsync(B->d_list, B->h_list.data(), B->h_list.size() * sizeof(int),
+                       cudaMemcpyHostToDevice, B->stream));
+    int max_nodes = 1;
+    for (int s : B->h_list) max_nodes = std::max(max_nodes, B->models[s]->n_nodes);
+    CL(launch_cluster_pack(B->d_sys, B->d_list, (int)B->h_list.size(), max_nodes, B->stream), 1);
+    const int steps = o->timeout_ms > 0.0 ? std::min(kClusterSteps, o->iters_per_launch)
+                                          : kClusterSteps;
+    const long long max_launches = (2LL * o->max_iter + 4LL * o->max_sweeps) / steps + 8;
+    for (long long launches = 1;; ++launches) {
+      sso_status st = launch_bins(B, bins, B->d_list, o->precond, steps);
+      if (st != SSO_OK) return st;
+      CK(cudaMemcpyAsync(B->h_flag + 2, B->d_n_active, 2 * sizeof(int), cudaMemcpyDeviceToHost,
+                         B->stream));
+      CK(cudaEventRecord(B->ev, B->stream));
+      CK(cudaEventSynchronize(B->ev));
+      if (B->h_flag[3] != 0)
+        return fail(SSO_ERR_CUDA, "CG kernel gave up waiting for a bulk copy (device fault?)");
+      if (B->h_flag[2] <= 0 || launches > max_launches) break;
+      if (o->timeout_ms > 0.0 && std::chrono::duration<double, std::milli>(
+                                     std::chrono::steady_clock::now() - t0).count() >
+                                     o->timeout_ms)
+        break;
+    }
   } else if (n_act > 0) {
     const bool two_level = o->precond == SSO_TWO_LEVEL;
     sso_status st = batch_graph(B, fp64, o->iters_per_launch, two_level);
@@ -1300,6 +1518,41 @@ TileDesc make_tile(const sso_model* M, int s, int k) {
   return d;
 }
 
+// One-cluster CG (cluster.cu): the extents of a CTA's share for every cluster
+// size, and whether the engine can take the structure at all: few enough
+// reduction chunks, and its padded copy of K no larger than the element-block
+// scratch it goes to.  Fixed by the mesh.
+void plan_cluster(sso_model* M, const HostTopo& T) {
+  const int n = M->n_nodes;
+  M->cl_positions = T.toff[M->n_tiles];
+  const size_t room = (size_t)std::max(M->n_eb, M->n_blocks) * 36 * sizeof(double);
+  M->cluster_ok = n_chunks_of(M) <= CL_MAX_CHUNKS && cluster_pack_bytes(M) <= room;
+  if (!M->cluster_ok) return;
+  for (int k = 0; k < CL_SIZES; ++k) {
+    const int C = cl_size_of(k);
+    int win = 0, pos = 0;
+    for (int r = 0; r < C; ++r) {  // the kernel's split of the tiles
+      const int t0 = (int)((long long)M->n_tiles * r / C);
+      const int t1 = (int)((long long)M->n_tiles * (r + 1) / C);
+      const int n0 = std::min(n, TILE * t0), n1 = std::min(n, TILE * t1);
+      int lo = n, hi = 0;
+      for (int i = n0; i < n1; ++i) {
+        lo = std::min(lo, T.col[T.row_ptr[i]]);
+        hi = std::max(hi, T.col[T.row_ptr[i + 1] - 1] + 1);
+      }
+      if (hi > lo) win = std::max(win, hi - lo);
+      pos = std::max(pos, T.toff[t1] - T.toff[t0]);
+    }
+    int members = 0;
+    for (int r = 0; r < C; ++r) {
+      int m = 0;
+      for (int g = r; g < T.n_agg; g += C) m += T.agg_ptr[g + 1] - T.agg_ptr[g];
+      members = std::max(members, m);
+    }
+    M->cl_share[k] = {M->n_tiles, (M->n_tiles + C - 1) / C, win, pos, members};
+  }
+}
+
 // Host half of a model: the mesh, validated, and its scatter map, node
 // incidence and tile descriptors, plus the packed image of every array the
 // device arena starts with.  Built without CUDA calls, so any thread may run
@@ -1409,6 +1662,16 @@ sso_status prepare_model(ModelPrep& P) {
         if (j == i + 1) Tm.chain_up[i] = b;
       }
   }
+  {  // block positions of every tile: its longest row
+    const int n = hm.n_nodes, nt = (n + TILE - 1) / TILE;
+    Tm.toff.assign(nt + 1, 0);
+    for (int t = 0; t < nt; ++t) {
+      int m = 0;
+      for (int i = t * TILE; i < std::min(n, (t + 1) * TILE); ++i)
+        m = std::max(m, Tm.row_ptr[i + 1] - Tm.row_ptr[i]);
+      Tm.toff[t + 1] = Tm.toff[t] + m;
+    }
+  }
   const HostTopo& T = P.T;
   sso_model* M = new sso_model();
   P.M = M;
@@ -1426,6 +1689,7 @@ sso_status prepare_model(ModelPrep& P) {
   M->h_row_ptr = T.row_ptr;
   M->h_col = T.col;
   sso_default_options(&M->last_opts);
+  plan_cluster(M, T);
   P.tiles.reserve(M->n_tiles);
   for (int t = 0; t < M->n_tiles; ++t) P.tiles.push_back(make_tile(M, -1, t));
   // every block's column slot in its tile's staged halo (the runs laid end
@@ -1482,6 +1746,7 @@ sso_status prepare_model(ModelPrep& P) {
   put(M->d_cg_ptr, T.cg_ptr.data(), T.cg_ptr.size() * 4);
   put(M->d_cg_src, T.cg_src.data(), T.cg_src.size() * 4);
   put(M->d_chain_up, T.chain_up.data(), T.chain_up.size() * 4);
+  put(M->d_toff, T.toff.data(), T.toff.size() * 4);
   {
     std::vector<double> e0(hm.n_quads), one(hm.n_quads, 1.0);
     for (int e = 0; e < hm.n_quads; ++e) e0[e] = hm.quad_props[5 * (size_t)e + 1];
@@ -1916,6 +2181,8 @@ sso_status create_batch(sso_model* const* models, int32_t n, sso_batch** out, bo
     D.cdot = M->d_cdot;
     D.zb = M->d_zb;
     D.klo = reinterpret_cast<float*>(M->d_ke);
+    D.toff = M->d_toff;
+    D.kc = reinterpret_cast<float*>(M->d_ke);
     for (int k = 0; k < M->n_tiles; ++k) tiles.push_back(make_tile(M, s, k));
   }
   B->n_tiles = (int)tiles.size();
@@ -2071,6 +2338,14 @@ void sso_batch_destroy(sso_batch* B) {
     cudaStreamDestroy(st);
   }
   for (cudaEvent_t e : B->aux_ev) cudaEventDestroy(e);
+  for (int k = 0; k < 2 * CL_SIZES - 1; ++k) {
+    if (B->cl_stream[k]) {
+      cudaStreamSynchronize(B->cl_stream[k]);
+      cudaStreamDestroy(B->cl_stream[k]);
+    }
+    if (B->cl_join[k]) cudaEventDestroy(B->cl_join[k]);
+  }
+  if (B->cl_fork) cudaEventDestroy(B->cl_fork);
   if (B->ev_fork) cudaEventDestroy(B->ev_fork);
   if (B->arena) cudaFree(B->arena);
   if (B->h_sc) cudaFreeHost(B->h_sc);
@@ -2674,6 +2949,8 @@ void fill_sysdesc(SysDesc& D, sso_model* M, int precond) {
   D.cdot = M->d_cdot;
   D.zb = M->d_zb;
   D.klo = reinterpret_cast<float*>(M->d_ke);
+  D.toff = M->d_toff;
+  D.kc = reinterpret_cast<float*>(M->d_ke);
 }
 
 void init_scalars(SysScalars& S, const sso_options& o) {

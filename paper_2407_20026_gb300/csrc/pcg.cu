@@ -157,27 +157,6 @@ __device__ __forceinline__ RunState read_state(const SysScalars* sc) {
   return r;
 }
 
-// Scalar update of kernel A for one system (one thread): sum = p^T q in a CG
-// iteration, else ||r64||^2; sum_b = ||b||^2.
-__device__ __forceinline__ void finish_a_scalars(SysScalars* sc, int state, double sum,
-                                                 double sum_b, int* n_active) {
-  if (state == ST_PCG) {
-    sc->pq = sum;
-    if (!(sum > 0.0) || !isfinite(sum)) {
-      sc->status = SSO_ERR_SINGULAR;
-      sc->state = ST_DONE;
-      atomicSub(n_active, 1);
-    } else {
-      sc->alpha = sc->rz / sum;
-      sc->parity ^= 1;
-    }
-  } else {
-    sc->rr64 = sum;
-    sc->ff = sum_b;
-  }
-  sc->cnt_a = 0u;
-}
-
 // Sums of the pairs p[2e], p[2e + 1] for e in [e0, min(e0 + CHUNK_PER_THREAD, e1)),
 // in e order; every load is issued before the first add.
 __device__ __forceinline__ void sum_pairs(const double* p, int e0, int e1, double& a,
@@ -382,66 +361,6 @@ __device__ __forceinline__ void st6(double* p, const double v[6]) {
   q[0] = make_double2(v[0], v[1]);
   q[1] = make_double2(v[2], v[3]);
   q[2] = make_double2(v[4], v[5]);
-}
-
-// Scalar update of kernel B for one system, by one thread, once every tile of
-// the system has been counted.  s1 = r^T z, s2 = r^T r.
-__device__ __forceinline__ void finish_b(SysScalars* sc, int state, double s1, double s2,
-                                         int* n_active, bool fold) {
-  if (state == ST_FOLD) {  // the correction has been added to x by every tile
-    sc->state = ST_RESID;
-  } else if (state == ST_PCG) {
-    sc->iters += 1;
-    sc->inner += 1;
-    if (!isfinite(s1) || !isfinite(s2)) {
-      sc->status = SSO_ERR_SINGULAR;
-      sc->state = ST_DONE;
-      atomicSub(n_active, 1);
-    } else {
-      sc->beta = s1 / sc->rz;
-      sc->rz = s1;
-      sc->rr = s2;
-      if (s2 <= sc->inner_thr || sc->iters >= sc->max_iter) sc->state = fold ? ST_FOLD : ST_RESID;
-    }
-  } else {
-    const double rr64 = sc->rr64;
-    if (!isfinite(rr64)) {
-      sc->status = SSO_ERR_INVALID;
-      sc->state = ST_DONE;
-      atomicSub(n_active, 1);
-    } else if (rr64 <= sc->rtol2 * sc->ff) {
-      sc->status = SSO_OK;
-      sc->state = ST_DONE;
-      atomicSub(n_active, 1);
-    } else if (sc->iters >= sc->max_iter || sc->sweeps >= sc->max_sweeps ||
-               (sc->sweeps >= 2 && rr64 > 0.0625 * sc->rr64_prev &&
-                !(sc->inner_rtol2 > 1e-12))) {
-      // cap reached, or the FP64 residual fell by less than 4x over the last
-      // sweep although the inner solve was already run to 1e-6 (rtol below
-      // what this K and FP64 can resolve)
-      sc->status = SSO_ERR_NOT_CONVERGED;
-      sc->state = ST_DONE;
-      atomicSub(n_active, 1);
-    } else if (!(s1 > 0.0)) {
-      sc->status = SSO_ERR_SINGULAR;  // preconditioner not positive definite
-      sc->state = ST_DONE;
-      atomicSub(n_active, 1);
-    } else {
-      // a sweep that gained less than 4x: the inner FP32 solve stopped before
-      // its own residual was trustworthy; run the following sweeps 10x tighter
-      if (sc->sweeps >= 2 && rr64 > 0.0625 * sc->rr64_prev) sc->inner_rtol2 *= 0.01;
-      sc->rz = s1;
-      sc->rr = s2;
-      sc->rr_start = s2;
-      sc->scale = ::sqrt(rr64);
-      sc->rr64_prev = rr64;
-      sc->inner_thr = s2 * fmax(sc->inner_rtol2, 0.25 * sc->rtol2 * sc->ff / rr64);
-      sc->inner = 0;
-      sc->sweeps += 1;
-      sc->state = ST_PCG;
-    }
-  }
-  sc->cnt_b = 0u;
 }
 
 // Two-level preconditioner: kernel B has only z_b = M_b^-1 r; it leaves

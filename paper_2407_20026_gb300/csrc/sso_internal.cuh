@@ -140,6 +140,10 @@ struct SysDesc {
   // double-float CG (precision SSO_F32X2, small.cu): the low parts of K,
   // K64 - K32 rounded to FP32, [n_blocks * 36] (the element-block scratch)
   float* klo;
+  // one-cluster CG (cluster.cu): block positions of the tiles [n_tiles + 1]
+  // (fixed by the mesh), K in that engine's layout (in the element-block scratch)
+  const int* toff;
+  float* kc;
   SysScalars* sc;
 };
 
@@ -258,6 +262,89 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t pari
   for (long long i = 0; i < kWaitPolls; ++i)
     if (mbar_test(bar, parity)) return true;
   return false;
+}
+
+// ---------------------------------------------------------------------------
+// Scalar updates of the CG's state machine (pcg.cu and cluster.cu).
+// Scalar update of kernel A for one system (one thread): sum = p^T q in a CG
+// iteration, else ||r64||^2; sum_b = ||b||^2.
+__device__ __forceinline__ void finish_a_scalars(SysScalars* sc, int state, double sum,
+                                                 double sum_b, int* n_active) {
+  if (state == ST_PCG) {
+    sc->pq = sum;
+    if (!(sum > 0.0) || !isfinite(sum)) {
+      sc->status = SSO_ERR_SINGULAR;
+      sc->state = ST_DONE;
+      atomicSub(n_active, 1);
+    } else {
+      sc->alpha = sc->rz / sum;
+      sc->parity ^= 1;
+    }
+  } else {
+    sc->rr64 = sum;
+    sc->ff = sum_b;
+  }
+  sc->cnt_a = 0u;
+}
+
+// Scalar update of kernel B for one system, by one thread, once every tile of
+// the system has been counted.  s1 = r^T z, s2 = r^T r.
+__device__ __forceinline__ void finish_b(SysScalars* sc, int state, double s1, double s2,
+                                         int* n_active, bool fold) {
+  if (state == ST_FOLD) {  // the correction has been added to x by every tile
+    sc->state = ST_RESID;
+  } else if (state == ST_PCG) {
+    sc->iters += 1;
+    sc->inner += 1;
+    if (!isfinite(s1) || !isfinite(s2)) {
+      sc->status = SSO_ERR_SINGULAR;
+      sc->state = ST_DONE;
+      atomicSub(n_active, 1);
+    } else {
+      sc->beta = s1 / sc->rz;
+      sc->rz = s1;
+      sc->rr = s2;
+      if (s2 <= sc->inner_thr || sc->iters >= sc->max_iter) sc->state = fold ? ST_FOLD : ST_RESID;
+    }
+  } else {
+    const double rr64 = sc->rr64;
+    if (!isfinite(rr64)) {
+      sc->status = SSO_ERR_INVALID;
+      sc->state = ST_DONE;
+      atomicSub(n_active, 1);
+    } else if (rr64 <= sc->rtol2 * sc->ff) {
+      sc->status = SSO_OK;
+      sc->state = ST_DONE;
+      atomicSub(n_active, 1);
+    } else if (sc->iters >= sc->max_iter || sc->sweeps >= sc->max_sweeps ||
+               (sc->sweeps >= 2 && rr64 > 0.0625 * sc->rr64_prev &&
+                !(sc->inner_rtol2 > 1e-12))) {
+      // cap reached, or the FP64 residual fell by less than 4x over the last
+      // sweep although the inner solve was already run to 1e-6 (rtol below
+      // what this K and FP64 can resolve)
+      sc->status = SSO_ERR_NOT_CONVERGED;
+      sc->state = ST_DONE;
+      atomicSub(n_active, 1);
+    } else if (!(s1 > 0.0)) {
+      sc->status = SSO_ERR_SINGULAR;  // preconditioner not positive definite
+      sc->state = ST_DONE;
+      atomicSub(n_active, 1);
+    } else {
+      // a sweep that gained less than 4x: the inner FP32 solve stopped before
+      // its own residual was trustworthy; run the following sweeps 10x tighter
+      if (sc->sweeps >= 2 && rr64 > 0.0625 * sc->rr64_prev) sc->inner_rtol2 *= 0.01;
+      sc->rz = s1;
+      sc->rr = s2;
+      sc->rr_start = s2;
+      sc->scale = ::sqrt(rr64);
+      sc->rr64_prev = rr64;
+      sc->inner_thr = s2 * fmax(sc->inner_rtol2, 0.25 * sc->rtol2 * sc->ff / rr64);
+      sc->inner = 0;
+      sc->sweeps += 1;
+      sc->state = ST_PCG;
+    }
+  }
+  sc->cnt_b = 0u;
 }
 
 #endif
@@ -415,6 +502,42 @@ cudaError_t launch_coarse_setup(int n_nodes, int n_agg, int n_blocks, const int*
                                 const uint8_t* fixed, const double* K64, double* node_r64,
                                 float* node_rf, double* T, double* Ac, float* W, float* Aci,
                                 cudaStream_t s);
+
+// One cluster of CTAs per system (cluster.cu).  Cluster sizes that fill the
+// GPCs well: 15 clusters of 9 CTAs are resident at once, as many as of 8, and
+// 23 of 6, 36 of 4; 7 of 16.
+constexpr int CL_SIZES = 7;
+constexpr int cl_size_of(int k) {
+  constexpr int size[CL_SIZES] = {1, 2, 3, 4, 6, 9, 16};
+  return size[k];
+}
+constexpr int CL_MAX_THREADS = 512;
+// CTAs of at most this many threads have the registers to keep CL_KREG
+// positions of K of every warp there (not with the two-level preconditioner).
+constexpr int CL_REG_THREADS = 384, CL_KREG = 1;
+constexpr int CL_POS_BYTES = 36 * 4 * 32;  // a block position of a tile
+constexpr int CL_MAX_CHUNKS = 4;      // of CHUNK tiles: systems of up to 30,720 nodes
+constexpr int CL_MAX_VWARPS = WARPS * CL_MAX_CHUNKS;
+// The largest share of a CTA: tiles of the system and of the CTA, nodes of
+// its window, block positions, members of its aggregates.
+struct ClusterShare {
+  int n_tiles, own_tiles, window, positions, members;
+};
+// Shared memory of a CTA without resident K; block positions that each of
+// `warps` warps keeps in tensor memory in a CTA of `smem` bytes (-1: no room).
+// m_tm: the preconditioner is there too.
+size_t cluster_smem_bytes(const ClusterShare& c, int precond, bool m_tm);
+int cluster_tm_positions(int smem, int own_tiles, int warps, bool m_tm);
+// The dynamic shared memory of a CTA and the clusters of each size that are
+// resident at once, with one CTA per SM.
+cudaError_t cluster_limits(int* max_smem, int slots[CL_SIZES]);
+cudaError_t launch_cluster_pack(const SysDesc* sys, const int* list, int n_list, int max_nodes,
+                                cudaStream_t s);
+// Systems list[0 .. n_list), one cluster of `size` CTAs each, up to max_steps
+// CG steps; flags[0] is lowered by each system that finishes.
+cudaError_t launch_cluster_cg(const SysDesc* sys, const int* list, int n_list, int size,
+                              int threads, int smem, int precond, bool m_tm, int* flags,
+                              int max_steps, cudaStream_t s);
 
 // Direct solve of a block-tridiagonal K by block cyclic reduction (chain.cu).
 // ws: chain_workspace_doubles(n) doubles; up[i]: index of block (i, i+1) in

@@ -1,0 +1,124 @@
+"""One-cluster CG (csrc/cluster.cu) against the two-kernel engine (csrc/pcg.cu).
+
+Both engines do the same arithmetic, so a solve must give the same bits, CG
+iterations and sweeps with either.  A profiled batch runs the two-kernel
+engine; sizes lie at the edges of tiles (30 nodes), of cluster sizes and of
+reduction chunks (256 tiles), and beyond what a cluster keeps on chip.  No
+tolerance: equality."""
+import numpy as np
+import pytest
+
+import meshgen
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sso():
+    import paper_2407_20026_gb300 as pkg
+    from paper_2407_20026_gb300 import _build
+    _build.build()
+    return pkg
+
+
+def _run(sso, meshes, profiled, g=None, **kw):
+    models = [sso.Model(m) for m in meshes]
+    batch = sso.Batch(models)
+    batch.set_profiling(profiled)
+    stats = batch.solve(sso.options(**kw), raise_on_error=False)
+    batch.gradient(g=g, raise_on_error=False)
+    batch.set_profiling(False)
+    return stats, [m.result() for m in models]
+
+
+def _same(sso, meshes, g=None, **kw):
+    a, ra = _run(sso, meshes, False, g, **kw)
+    b, rb = _run(sso, meshes, True, g, **kw)
+    for x, y, p, q in zip(a, b, ra, rb):
+        for k in ("status", "iterations", "sweeps", "rel_residual"):
+            assert x[k] == y[k], (k, x, y)
+        for k in ("u", "C", "dz", "dt", "lam"):
+            assert np.array_equal(p[k], q[k]), k
+    return a
+
+
+def _strip(n):
+    """A clamped-free beam line of n nodes, numbered along it (n = 30 k + r)."""
+    m = meshgen.arch2d(n_el=n - 1, E=2e11)
+    m["xyz"][:, 1] = 0.1 * np.sin(np.arange(n))
+    return m
+
+
+@pytest.mark.parametrize("precond", ["jacobi", "block_jacobi", "two_level"])
+@pytest.mark.parametrize("n", [2, 29, 30, 31, 61])
+def test_tile_edges(sso, n, precond):
+    _same(sso, [_strip(n)], precond=precond, rtol=1e-6, max_iter=400)
+
+
+@pytest.mark.parametrize("precond", ["jacobi", "block_jacobi", "two_level"])
+@pytest.mark.parametrize("size", [3, 8, 19, 33, 64])
+def test_shells(sso, size, precond):
+    # 16 to 4,225 nodes: one to sixteen CTAs, K resident or through L2
+    _same(sso, [meshgen.shell(size, seed=size)], precond=precond, rtol=1e-6, max_iter=3000)
+
+
+@pytest.mark.parametrize("precond", ["block_jacobi", "two_level"])
+@pytest.mark.parametrize("side", [87, 88, 100])
+def test_reduction_chunks(sso, side, precond):
+    # 7,569, 7,744 and 10,000 nodes: 253, 259 and 334 tiles, one and two chunks
+    _same(sso, [meshgen.gridshell(side, seed=side)], precond=precond, rtol=1e-6, max_iter=700)
+
+
+def test_scattered_numbering_and_hub(sso):
+    # windows as wide as the system; one row of as many blocks as it has nodes
+    m = meshgen.gridshell(17, seed=4)
+    rng = np.random.default_rng(5)
+    perm = rng.permutation(m["xyz"].shape[0])
+    inv = np.argsort(perm)
+    m["beam_conn"] = inv[m["beam_conn"]].astype(np.int32)
+    for k in ("xyz", "fixed", "nodal_load"):
+        m[k] = m[k][perm]
+    _same(sso, [m], rtol=1e-6)
+    h = meshgen.gridshell(9, seed=6)
+    hub = 40
+    far = np.array([j for j in range(81) if j not in (hub,) and (j // 9 + j) % 3 == 0], np.int32)
+    have = {tuple(sorted(c)) for c in h["beam_conn"].tolist()}
+    new = np.array([(hub, j) for j in far if tuple(sorted((hub, int(j)))) not in have], np.int32)
+    h["beam_conn"] = np.concatenate([h["beam_conn"], new])
+    h["beam_props"] = np.tile(h["beam_props"][0], (h["beam_conn"].shape[0], 1))
+    _same(sso, [h], rtol=1e-6)
+
+
+def test_mixed_batch_more_systems_than_clusters_and_adjoint(sso):
+    meshes = [meshgen.shell(20, seed=1), meshgen.gridshell(10), meshgen.gridshell(50, seed=2),
+              meshgen.shell(7)] + [meshgen.shell(33, seed=s) for s in range(20)]
+    rng = np.random.default_rng(9)
+    g = [rng.standard_normal(6 * m["xyz"].shape[0]) * (k % 2) for k, m in enumerate(meshes)]
+    _same(sso, meshes, g=g, rtol=1e-6, max_iter=4000)
+
+
+def test_many_launches_and_caps(sso):
+    # a wall-clock cap launches iters_per_launch steps at a time: the state
+    # passes through memory between launches, also in the middle of a sweep
+    m = meshgen.shell(12, seed=3)
+    whole = _run(sso, [m], False, rtol=1e-8)
+    for n in (1, 7, 64):
+        cut = _run(sso, [m], False, rtol=1e-8, timeout_ms=6e4, iters_per_launch=n)
+        assert cut[0][0]["iterations"] == whole[0][0]["iterations"]
+        assert np.array_equal(cut[1][0]["u"], whole[1][0]["u"])
+    two = [_run(sso, [m], False, rtol=1e-8, precond="two_level", **kw)
+           for kw in ({}, {"timeout_ms": 6e4, "iters_per_launch": 5})]
+    assert np.array_equal(two[0][1][0]["u"], two[1][1][0]["u"])
+    _same(sso, [m], rtol=1e-8, max_iter=50)
+    _same(sso, [m], rtol=1e-8, max_sweeps=1)
+
+
+def test_zero_load_mechanism_and_warm_start(sso):
+    m = meshgen.gridshell(10)
+    z = dict(m, nodal_load=np.zeros_like(m["nodal_load"]))
+    assert _same(sso, [z], rtol=1e-8)[0]["iterations"] == 0
+    free = dict(m, fixed=np.zeros_like(m["fixed"]))
+    assert _same(sso, [free], rtol=1e-8, max_iter=2000)[0]["status"] != 0
+    mdl = sso.Model(m)
+    mdl.solve(rtol=1e-4)
+    assert mdl.solve(rtol=1e-8, warm_start=1)["status"] == 0
