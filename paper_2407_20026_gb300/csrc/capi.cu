@@ -1072,13 +1072,6 @@ sso_status cluster_device(const ClusterDevice** out) {
   return SSO_OK;
 }
 
-// Warps of a CTA: as few rounds of tiles per warp as the limit allows, evenly
-// filled.
-int cluster_warps(int own_tiles) {
-  const int most = CL_MAX_THREADS / 32, rounds = (own_tiles + most - 1) / most;
-  return std::max(2, (own_tiles + rounds - 1) / rounds);
-}
-
 // How a structure runs when n_sys run together: the cluster size (index; -1:
 // the two-kernel engine), and whether tensor memory holds the preconditioner.
 // The least estimated time of all n_sys: an iteration is the barriers,

@@ -641,7 +641,10 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
   const SysDesc& S = sh.sys;
   const int n = S.n_nodes, n_tiles = S.n_tiles, n_ow = WARPS * n_tiles;
   const int T0 = n_tiles * (int)rank / (int)C, T1 = n_tiles * ((int)rank + 1) / (int)C;
-  const int nt = T1 - T0, W = min(nth >> 5, max(nt, 1));  // W: warps that own tiles
+  // W: warps that own tiles, the system's own number (a launch may have more,
+  // for another system of its list: the plan counts slots of K for this many)
+  const int nt = T1 - T0;
+  const int W = min(min(nth >> 5, cluster_warps((n_tiles + (int)C - 1) / (int)C)), max(nt, 1));
   const int n0 = min(n, TILE * T0), n1 = min(n, TILE * T1), nown = n1 - n0;
   const int U0 = __ldg(S.toff + T0), U1 = __ldg(S.toff + T1);
   {  // the nodes that this CTA's rows read
@@ -787,12 +790,13 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
     for (int i = tid; i < 3 * nown; i += nth) reinterpret_cast<float2*>(Ms)[i] = __ldg(m2 + i);
   }
   // This warp's tiles are contiguous, so its K is one run of m positions: the
-  // first nkr in registers (CTAs of few warps), the next ntm in tensor memory (the
-  // warp's share of its quadrant's columns), the ns others through its cap slots of shared memory.  Where these do not all
-  // fit, the slots are a ring that bulk copies refill from L2: the k-th use of
-  // the ring is the k mod ns-th of them, in slot k mod cap, and a consumed slot
-  // takes the one cap uses on, so that the copies run ahead of the products,
-  // through the barriers and into the next iteration.
+  // first nkr in registers (CTAs of few warps), the next ntm in tensor memory
+  // (the warp's share of its quadrant's columns), the ns others through its cap
+  // slots of shared memory (at least one: the plan's rule).  Where these do not
+  // all fit, the slots are a ring that bulk copies refill from L2: the k-th use
+  // of the ring is the k mod ns-th of them, in slot k mod cap, and a consumed
+  // slot takes the one cap uses on, so that the copies run ahead of the
+  // products, through the barriers and into the next iteration.
   const int ta = w < W ? T0 + nt * w / W : T1, tb = w < W ? T0 + nt * (w + 1) / W : T1;
   const int pa = __ldg(S.toff + ta), m = __ldg(S.toff + tb) - pa;
   if (tm_cols && w == 0) tm_alloc(&sh.tmem, tm_cols);
@@ -813,6 +817,7 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
       }
     }
   const int nkr = min(m, KREG), ntm = min(m - nkr, (tm_share - tm_m) / 36), ns = cap ? m - nkr - ntm : 0;
+  if (ns < m - nkr - ntm && lane == 0) atomicExch(flags + 1, 1);  // no launch of the plan's
   Kg += (size_t)nkr * CL_POS_F4;
   const uint32_t tmw =
       tm_cols ? sh.tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)((w >> 2) * tm_share) : 0u;
@@ -979,7 +984,7 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
           }
         __syncwarp();
 #pragma unroll 1
-        for (int i = 0; i < m - nkr; ++i) {
+        for (int i = 0; i < ntm + ns; ++i) {
           KPos K;
           float p[6];
           load(K, i);

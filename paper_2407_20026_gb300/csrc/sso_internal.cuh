@@ -512,6 +512,13 @@ constexpr int cl_size_of(int k) {
   return size[k];
 }
 constexpr int CL_MAX_THREADS = 512;
+// Warps that own a CTA's tiles: as few rounds of tiles per warp as the limit
+// allows, evenly filled.
+__host__ __device__ constexpr int cluster_warps(int own_tiles) {
+  const int most = CL_MAX_THREADS / 32, rounds = (own_tiles + most - 1) / most;
+  const int even = rounds > 0 ? (own_tiles + rounds - 1) / rounds : 0;
+  return even > 2 ? even : 2;
+}
 // CTAs of at most this many threads have the registers to keep CL_KREG
 // positions of K of every warp there (not with the two-level preconditioner).
 constexpr int CL_REG_THREADS = 384, CL_KREG = 1;

@@ -97,6 +97,13 @@ def test_mixed_batch_more_systems_than_clusters_and_adjoint(sso):
     _same(sso, meshes, g=g, rtol=1e-6, max_iter=4000)
 
 
+@pytest.mark.parametrize("precond", ["jacobi", "block_jacobi", "two_level"])
+def test_launches_of_systems_with_different_warps(sso, precond):
+    # one launch's CTAs have the warps of its largest system
+    meshes = [meshgen.gridshell(side, seed=side) for side in range(31, 101, 3)]
+    _same(sso, meshes, precond=precond, rtol=1e-6, max_iter=300)
+
+
 def test_many_launches_and_caps(sso):
     # a wall-clock cap launches iters_per_launch steps at a time: the state
     # passes through memory between launches, also in the middle of a sweep
