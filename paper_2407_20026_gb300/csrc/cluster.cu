@@ -69,10 +69,17 @@ __device__ __forceinline__ unsigned cl_size() {
 }
 // Barrier over every thread of the cluster; orders shared (own and remote) and
 // global memory accesses of the threads on both sides.
-__device__ __forceinline__ void cl_sync() {
+__device__ __forceinline__ void cl_arrive() {
   __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cl_wait() {
+  __syncwarp();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cl_sync() {
+  cl_arrive();
+  cl_wait();
 }
 __device__ __forceinline__ uint32_t cl_map(uint32_t addr, unsigned rank) {
   uint32_t r;
@@ -625,6 +632,7 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
   {
     const SysDesc& G = sys[list[blockIdx.x / C]];
     if (*(volatile const int*)&G.sc->state == ST_DONE) return;  // alike in every CTA
+    cl_arrive();  // waited for before the first store to another CTA
 #pragma unroll 1
     for (int i = tid; i < (int)(sizeof(SysDesc) / 4); i += nth)
       reinterpret_cast<int*>(&sh.sys)[i] = reinterpret_cast<const int*>(&G)[i];
@@ -875,12 +883,15 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
   float beta = (float)sh.sc.beta;
   int kA = 0, kB = kGrid - f64_exp(sh.sc.rz), kR = kGrid - f64_exp(sh.sc.rr), par = 0;
   bool have_kA = false;
-  // every CTA has read the system's state and may receive stores from here on
+  // Every CTA has started by now (one that has not must not be stored to: the
+  // CTAs of a cluster are placed together, but an SM that has to drain another
+  // kernel first starts its own late) ...
+  cl_wait();
   if (tid < (int)C) {
     cl_st(cl_map(smem_addr(&sh.wlo[rank]), tid), lo);
     cl_st(cl_map(smem_addr(&sh.whi[rank]), tid), lo + wn);
   }
-  cl_sync();
+  cl_sync();  // ... and has read the system's state and set up its windows
   unsigned dest = 0u;  // CTAs whose windows reach this warp's nodes
 #pragma unroll 1
   for (unsigned c = 0; c < C; ++c)
