@@ -1136,9 +1136,10 @@ ClusterChoice cluster_choice(const sso_model* M, int n_sys, int precond,
 
 // Sorts the active systems into launches by cluster size; *fits is false when
 // a system does not fit the engine (the batch then runs the two-kernel engine).
+// sharers: batches of about as many systems on the device at the same time.
 template <class GetModel>
-sso_status plan_bins(int n_sys, const std::vector<char>& active, int precond, GetModel model,
-                     std::vector<int>& list, std::vector<ClusterBin>& bins, bool* fits) {
+sso_status plan_bins(int n_sys, const std::vector<char>& active, int precond, int sharers,
+                     GetModel model, std::vector<int>& list, std::vector<ClusterBin>& bins, bool* fits) {
   *fits = false;
   list.clear();
   bins.clear();
@@ -1150,7 +1151,7 @@ sso_status plan_bins(int n_sys, const std::vector<char>& active, int precond, Ge
   std::vector<ClusterChoice> choice(n_sys);
   for (int s = 0; s < n_sys; ++s) {
     if (!active[s]) continue;
-    choice[s] = cluster_choice(model(s), n_act, precond, *dev);
+    choice[s] = cluster_choice(model(s), n_act * sharers, precond, *dev);
     if (choice[s].size < 0) return SSO_OK;
   }
   for (int k = CL_SIZES - 1; k >= 0; --k)
@@ -1229,7 +1230,7 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
   bool cluster = false;
   std::vector<ClusterBin> bins;
   if (o->precision == SSO_FP32_IR && !B->profiling) {
-    sso_status st = plan_bins(B->n_sys, active, o->precond,
+    sso_status st = plan_bins(B->n_sys, active, o->precond, 1,
                               [B](int s) { return B->models[s]; }, B->h_list, bins, &cluster);
     if (st != SSO_OK) return st;
   }
@@ -2711,6 +2712,7 @@ sso_status batch_with_capacity(cudaStream_t stream, int max_sys, int max_tiles,
   c.take<AggRef>((size_t)max_sys * COARSE_MAX_AGG);
   c.take<int>(max_sys);
   c.take<int>(2);
+  c.take<int>(2 * (size_t)max_sys);
   const size_t bytes = align_up(c.off, 256);
   cudaError_t e = cudaMalloc(&B->arena, bytes);
   if (e != cudaSuccess) {
@@ -2729,6 +2731,7 @@ sso_status batch_with_capacity(cudaStream_t stream, int max_sys, int max_tiles,
   B->d_aggs = d.take<AggRef>((size_t)max_sys * COARSE_MAX_AGG);
   B->d_csys = d.take<int>(max_sys);
   B->d_ccount = d.take<int>(2);
+  B->d_list = d.take<int>(2 * (size_t)max_sys);  // clusters' systems; systems to pack
   B->n_aggs = max_sys * COARSE_MAX_AGG;
   {
     int dev = 0, sms = 0;
@@ -2778,6 +2781,11 @@ struct sso_server {
   std::vector<int> running, pending;
   std::vector<std::vector<TileDesc>> slot_tiles;  // tile descriptors of each slot's model
   int tiles_used = 0;  // tiles of running + pending systems
+  // launches of the cluster engine for the running systems (empty: the
+  // two-kernel graph), and the slots whose K is packed for it
+  std::vector<ClusterBin> bins;
+  std::vector<char> packed;
+  int lane_count = 1;  // servers that share the device's clusters
   uint64_t next_ticket = 1;
   std::chrono::steady_clock::time_point t0;
   bool dirty = false;
@@ -2819,6 +2827,12 @@ struct sso_server {
 
 namespace {
 constexpr int kIdleAdmit = 16;  // requests admitted per step while no CG graph runs
+// CG steps of a system per launch of the cluster engine, in graphs' worth of
+// iterations: its iterations take about half the graph's time, and a launch
+// loads the systems anew.  64 grid shells of sides 8 to 100, two lanes, ms: 151
+// with 1, 143 with 2, 138 with 4, 136 with 8, 140 with 16; 8 of sides 8 to 40:
+// 8.9, 8.4, 8.2, 8.6, 9.9 (a system that finishes waits for the launch's end).
+constexpr int kServerRounds = 4;
 constexpr int kSetupStreams = 8;  // set-up streams of a server
 constexpr size_t kRingBytes = 64u << 20;  // pinned upload staging of a server
 
@@ -2900,6 +2914,37 @@ sso_status server_upload_tables(sso_server* S, std::vector<std::vector<TileDesc>
   CK(cudaMemcpyAsync(B->d_ccount, ccount, sizeof(ccount), cudaMemcpyHostToDevice, B->stream));
   CK(cudaMemcpyAsync(B->d_sys, B->h_sys.data(), sizeof(SysDesc) * S->max_sys,
                      cudaMemcpyHostToDevice, B->stream));
+  // one cluster per system while every running system fits (the engines'
+  // results are the same bits, and each takes over the other's state)
+  S->bins.clear();
+  std::vector<int> pack;
+  if (S->opts.precision == SSO_FP32_IR && !S->running.empty()) {
+    std::vector<char> active(S->max_sys, 0);
+    for (int slot : S->running) active[slot] = 1;
+    bool fits = false;
+    sso_status st = plan_bins(S->max_sys, active, S->opts.precond, S->lane_count,
+                              [S](int slot) { return S->slot_req[slot]->M; }, B->h_list,
+                              S->bins, &fits);
+    if (st != SSO_OK) return st;
+    if (!fits) S->bins.clear();
+    if (fits) {
+      int max_nodes = 1;
+      for (int slot : S->running)
+        if (!S->packed[slot]) {
+          pack.push_back(slot);
+          max_nodes = std::max(max_nodes, S->slot_req[slot]->M->n_nodes);
+          S->packed[slot] = 1;
+        }
+      CK(cudaMemcpyAsync(B->d_list, B->h_list.data(), B->h_list.size() * sizeof(int),
+                         cudaMemcpyHostToDevice, B->stream));
+      if (!pack.empty()) {
+        int* d_pack = B->d_list + S->max_sys;
+        CK(cudaMemcpyAsync(d_pack, pack.data(), pack.size() * sizeof(int),
+                           cudaMemcpyHostToDevice, B->stream));
+        CL(launch_cluster_pack(B->d_sys, d_pack, (int)pack.size(), max_nodes, B->stream), 1);
+      }
+    }
+  }
   CK(cudaStreamSynchronize(B->stream));  // the host vectors above are temporaries
   S->dirty = false;
   return SSO_OK;
@@ -3056,6 +3101,7 @@ sso_status sso_server_create_lanes(const sso_options* opts, size_t hbm_budget_by
       delete S;
       return st;
     }
+    L->lane_count = lanes;
     S->lanes.push_back(L);
   }
   S->global_of.resize(lanes);
@@ -3095,6 +3141,7 @@ sso_status sso_server_create(const sso_options* opts, size_t hbm_budget_bytes,
   S->max_tiles = max_tiles;
   S->slot_req.assign(max_systems, nullptr);
   S->slot_tiles.assign(max_systems, {});
+  S->packed.assign(max_systems, 0);
   S->t0 = std::chrono::steady_clock::now();
   const unsigned hw = std::thread::hardware_concurrency();
   const int n_workers = (int)std::min(8u, std::max(1u, hw));
@@ -3231,9 +3278,15 @@ sso_status sso_server_step(sso_server* S, int32_t* n_running, int32_t* n_waiting
     B->h_flag[1] = 0;
     CK(cudaMemcpyAsync(B->d_n_active, B->h_flag, 2 * sizeof(int), cudaMemcpyHostToDevice,
                        B->stream));
-    if ((st = batch_graph(B, fp64, iters, two_level)) != SSO_OK) return st;
-    CK(cudaGraphLaunch(B->exec[k], B->stream));
-    g_launches += (two_level ? 5ull : 2ull) * (unsigned long long)iters;
+    if (!S->bins.empty()) {
+      if ((st = launch_bins(B, S->bins, B->d_list, S->opts.precond,
+                            kServerRounds * iters)) != SSO_OK)
+        return st;
+    } else {
+      if ((st = batch_graph(B, fp64, iters, two_level)) != SSO_OK) return st;
+      CK(cudaGraphLaunch(B->exec[k], B->stream));
+      g_launches += (two_level ? 5ull : 2ull) * (unsigned long long)iters;
+    }
     if ((st = debug_check(B->stream, "server: CG graph")) != SSO_OK) return st;
     CK(cudaMemcpyAsync(B->h_flag + 2, B->d_n_active, 2 * sizeof(int), cudaMemcpyDeviceToHost,
                        B->stream));
@@ -3351,6 +3404,7 @@ sso_status sso_server_step(sso_server* S, int32_t* n_running, int32_t* n_waiting
     R->slot = slot;
     R->phase = 1;
     S->slot_req[slot] = R;
+    S->packed[slot] = 0;
     S->slot_tiles[slot].swap(R->prep->tiles);
     for (TileDesc& td : S->slot_tiles[slot]) td.sys = slot;
     R->prep.reset();

@@ -129,3 +129,28 @@ def test_zero_load_mechanism_and_warm_start(sso):
     mdl = sso.Model(m)
     mdl.solve(rtol=1e-4)
     assert mdl.solve(rtol=1e-8, warm_start=1)["status"] == 0
+
+
+def test_server_switches_engines(sso):
+    # a system beyond the engine's size joins and leaves while others run: the
+    # server's running systems change engines in the middle of their sweeps
+    from paper_2407_20026_gb300.serve import Server
+    opts = sso.options(rtol=1e-4)
+    small = [meshgen.gridshell(side, seed=side) for side in (60, 30, 90, 45, 20, 100)]
+    large = meshgen.gridshell(176, seed=1)  # 30,976 nodes: five reduction chunks
+    srv = Server(opts, max_systems=8)
+    tickets = [srv.submit(m) for m in small[:3]]
+    for _ in range(3):
+        srv.step()
+    tickets.append(srv.submit(large))
+    tickets += [srv.submit(m) for m in small[3:]]
+    while any(srv.step()):
+        pass
+    for m, t in zip(small[:3] + [large] + small[3:], tickets):
+        mdl = sso.Model(m)
+        mdl.solve(opts)
+        mdl.gradient()
+        want, got = mdl.result(), srv.poll(t)
+        assert got["stats"]["status"] == 0
+        assert np.array_equal(got["u"], want["u"]) and got["C"] == want["C"]
+    srv.close()
