@@ -222,7 +222,7 @@ __device__ __forceinline__ void fma_pos(const KPos& k, const float* p,
 // A partial of a CG sum, or several, on an integer grid (below).
 struct Fix {
   long long s;    // on the grid
-  unsigned a;     // magnitude >> 32, rounded up
+  unsigned a;     // magnitude >> 38, rounded up
   unsigned bad;   // not finite, or 2 times the previous sum and more
 };
 // A positive value (h + l) 2^e, h in [1, 2), to about 2^-47.
@@ -295,7 +295,7 @@ __device__ __forceinline__ Fix to_fix(DF x, int k) {
   Fix f;
   f.bad = 0u;
   f.s = fix_part(x.hi, k, f.bad) + fix_part(x.lo, k, f.bad);
-  f.a = (unsigned)((f.s < 0 ? -f.s : f.s) >> 32) + 1u;
+  f.a = (unsigned)((f.s < 0 ? -f.s : f.s) >> 38) + 1u;  // (at most 2^14: no sum overflows)
   return f;
 }
 // Sum over the warp, in every lane.
@@ -343,7 +343,7 @@ __device__ __forceinline__ Apx apx_f64(double x) {  // positive and finite (a su
 // The sum on the grid 2^-k; false where its bound does not hold.
 __device__ __forceinline__ bool apx_fix(const Fix& f, int k, Apx& out) {
   if (f.bad || f.s < (1ll << (kGrid - 1)) || f.s >= (1ll << (kGrid + 3)) ||
-      (f.a >> 10) > (unsigned)(f.s >> 32))
+      (long long)f.a > f.s >> 28)
     return false;
   const int lz = __clzll(f.s);
   out = apx_bits((unsigned long long)f.s << lz, 63 - lz - k);
@@ -367,7 +367,7 @@ __device__ __forceinline__ bool apx_quotient(const Apx& a, const Apx& b, float& 
          half - fabsf(rest) > 0x1p-34f;
 }
 // value <= thr for the sum f on the grid 2^-k; sets *clear where the bounds
-// leave no doubt.
+// leave no doubt (the sum's own is 2^-33 of it).
 __device__ __forceinline__ bool fix_le(const Fix& f, int k, double thr, bool& clear) {
   const long long b = __double_as_longlong(thr);
   const int sh = (int)(b >> 52) - 1075 + k;  // thr = m 2^(sh - k)
@@ -462,7 +462,9 @@ __device__ __noinline__ void exact_sums(ClShared& sh, int par, bool with_a) {
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, W = blockDim.x >> 5;
   const int n_tiles = sh.sys.n_tiles, n_ow = sh.n_ow, n_chunks = sh.sys.n_chunks;
   const int n_vw = (n_ow + 255) / 256;
-  double *bufA = sh.sys.part_a, *bufB = sh.sys.part_b;
+  // (a buffer of r^T z and r^T r per parity: the sums of the previous iteration
+  // and of this one are formed one after the other, with no barrier between)
+  double *bufA = sh.sys.part_a, *bufB = sh.sys.part_b + 2 * (size_t)n_tiles * par;
 #pragma unroll 1
   for (int t = tid; t < sh.nt; t += blockDim.x) {
     const float4 v = sh.tB[par * sh.nt + t];
