@@ -236,7 +236,7 @@ struct sso_model {
   // size the largest share of a CTA
   bool cluster_ok = false;
   int cl_positions = 0;
-  ClusterShare cl_share[CL_SIZES] = {};
+  ClusterShare cl_share[CL_SIZES] = {}, cl_team[CL_TEAMS] = {};
   int* d_toff;
   bool is_chain = false;
   int* d_chain_up;        // [n_nodes] block (i, i+1) or -1
@@ -315,6 +315,7 @@ struct sso_batch {
   // SSO_F32X2: the systems being solved (one CTA each); one-cluster CG: the
   // systems by cluster size
   int* d_list = nullptr;
+  unsigned long long* d_slots = nullptr;  // CL_SLOT_BYTES: the teams' barrier words
   std::vector<int> h_list;
   // one-cluster CG: extra streams for the launches of further cluster sizes
   cudaStream_t cl_stream[2 * CL_SIZES - 1] = {};
@@ -1053,11 +1054,12 @@ sso_status finish_run(sso_batch* B, const std::vector<char>& active, sso_stats* 
 struct ClusterBin {
   int first, n, size, threads, smem;
   bool m_tm;  // the preconditioner in tensor memory
+  bool team;  // teams of a cooperative launch, not clusters
 };
 
 // What the device holds at once (cluster_limits).
 struct ClusterDevice {
-  int smem = 0, slots[CL_SIZES];
+  int smem = 0, slots[CL_SIZES], ctas = 0;
 };
 sso_status cluster_device(const ClusterDevice** out) {
   static std::mutex mu;
@@ -1065,7 +1067,7 @@ sso_status cluster_device(const ClusterDevice** out) {
   std::lock_guard<std::mutex> lock(mu);
   if (!d.smem) {
     ClusterDevice q;
-    CK(cluster_limits(&q.smem, q.slots));
+    CK(cluster_limits(&q.smem, q.slots, &q.ctas));
     d = q;
   }
   *out = &d;
@@ -1086,19 +1088,25 @@ sso_status cluster_device(const ClusterDevice** out) {
 // iteration, where the two-kernel engine is as fast.
 constexpr size_t kClusterL2 = (size_t)100 << 20;
 constexpr double kClusterFixed = 9500.0, kClusterRound = 5000.0;
+// Teams (cooperative launches), us an iteration, cluster -> team where either
+// runs: 72 x 72 shell 8.5 -> 8.5, 80 x 80 9.8 -> 8.9, grid shell of 80 x 80
+// nodes 8.3 -> 8.3, of 90 x 90 12.2 -> 8.3; 64 x 64 shell 7.1 -> 9.4.  Teams
+// need a tile per CTA.
+constexpr double kTeamFixed = 11500.0;
 struct ClusterChoice {
   int size = -1;
-  bool m_tm = false;
+  bool m_tm = false, team = false;
 };
-ClusterChoice cluster_choice(const sso_model* M, int n_sys, int precond,
+ClusterChoice cluster_choice(const sso_model* M, int n_sys, int precond, bool teams,
                              const ClusterDevice& d) {
   ClusterChoice best;
   if (!M->cluster_ok) return best;
   double best_t = HUGE_VAL;
-  for (int k = 0; k < CL_SIZES; ++k) {
-    const ClusterShare& sh = M->cl_share[k];
-    const int C = cl_size_of(k), slots = d.slots[k], warps = cluster_warps(sh.own_tiles);
-    if (slots < 1 || sh.window >= 65535 || (k > 0 && M->n_tiles < 2 * C)) continue;
+  auto consider = [&](bool team, int k) {
+    const ClusterShare& sh = team ? M->cl_team[k] : M->cl_share[k];
+    const int C = team ? cl_team_of(k) : cl_size_of(k);
+    const int slots = team ? std::min(d.ctas / C, CL_MAX_TEAMS) : d.slots[k], warps = cluster_warps(sh.own_tiles);
+    if (slots < 1 || sh.window >= 65535 || (C > 1 && M->n_tiles < (team ? C : 2 * C))) return;
     // The preconditioner in shared memory, or in tensor memory (CTAs that use
     // all of their shared memory anyway), whichever leaves less of K to L2; a
     // position of K per warp in shared memory at least: the ring behind L2.
@@ -1108,7 +1116,7 @@ ClusterChoice cluster_choice(const sso_model* M, int n_sys, int precond,
     size_t stream = SIZE_MAX;
     bool m_tm = false;
     for (int in_tm = 0; in_tm < (precond == SSO_JACOBI ? 1 : 2); ++in_tm) {
-      const size_t need = cluster_smem_bytes(sh, precond, in_tm);
+      const size_t need = cluster_smem_bytes(sh, precond, in_tm, team);
       const int pos = cluster_tm_positions(d.smem, sh.own_tiles, warps, in_tm);
       if (pos < 0 || need + (size_t)CL_POS_BYTES * warps > (size_t)d.smem ||
           (in_tm && need + share <= (size_t)d.smem))
@@ -1120,26 +1128,33 @@ ClusterChoice cluster_choice(const sso_model* M, int n_sys, int precond,
         m_tm = in_tm;
       }
     }
-    if (stream == SIZE_MAX) continue;
-    if ((size_t)std::min(slots, n_sys) * C * stream > kClusterL2) continue;
+    if (stream == SIZE_MAX) return;
+    if ((size_t)std::min(slots, n_sys) * C * stream > kClusterL2) return;
     const double rounds = (double)sh.own_tiles / warps;
-    const double t = kClusterFixed + kClusterRound * rounds + stream / 64.0;
-    const double waves = n_sys <= slots ? 1.0 : (double)n_sys / slots;
+    const double t = (team ? kTeamFixed : kClusterFixed) + kClusterRound * rounds + stream / 64.0;
+    const double waves = n_sys <= slots ? 1.0
+                         : team         ? (double)((n_sys + slots - 1) / slots)
+                                        : (double)n_sys / slots;
     if (t * waves < best_t) {
       best_t = t * waves;
       best.size = k;
       best.m_tm = m_tm;
+      best.team = team;
     }
-  }
+  };
+  for (int k = 0; k < CL_SIZES; ++k) consider(false, k);
+  if (teams && precond != SSO_TWO_LEVEL)
+    for (int k = 0; k < CL_TEAMS; ++k) consider(true, k);
   return best;
 }
 
 // Sorts the active systems into launches by cluster size; *fits is false when
 // a system does not fit the engine (the batch then runs the two-kernel engine).
-// sharers: batches of about as many systems on the device at the same time.
+// sharers: batches of about as many systems on the device at the same time;
+// teams: cooperative launches may be used.
 template <class GetModel>
 sso_status plan_bins(int n_sys, const std::vector<char>& active, int precond, int sharers,
-                     GetModel model, std::vector<int>& list, std::vector<ClusterBin>& bins, bool* fits) {
+                     bool teams, GetModel model, std::vector<int>& list, std::vector<ClusterBin>& bins, bool* fits) {
   *fits = false;
   list.clear();
   bins.clear();
@@ -1151,58 +1166,87 @@ sso_status plan_bins(int n_sys, const std::vector<char>& active, int precond, in
   std::vector<ClusterChoice> choice(n_sys);
   for (int s = 0; s < n_sys; ++s) {
     if (!active[s]) continue;
-    choice[s] = cluster_choice(model(s), n_act * sharers, precond, *dev);
+    choice[s] = cluster_choice(model(s), n_act * sharers, precond, teams, *dev);
     if (choice[s].size < 0) return SSO_OK;
   }
-  for (int k = CL_SIZES - 1; k >= 0; --k)
-    for (int m_tm = 0; m_tm < 2; ++m_tm) {
-      ClusterBin b{(int)list.size(), 0, cl_size_of(k), 0, 0, m_tm != 0};
-      for (int s = 0; s < n_sys; ++s) {
-        if (choice[s].size != k || choice[s].m_tm != b.m_tm) continue;
-        const ClusterShare& sh = model(s)->cl_share[k];
-        // all of a CTA's K resident where it fits, else whatever room is left
-        const size_t all = m_tm ? dev->smem
-                                : cluster_smem_bytes(sh, precond, false) +
-                                      (size_t)CL_POS_BYTES * (sh.positions + 2);
-        b.smem = std::max(b.smem, (int)std::min((size_t)dev->smem, all));
-        b.threads = std::max(b.threads, 32 * cluster_warps(sh.own_tiles));
-        list.push_back(s);
-        ++b.n;
-      }
-      if (b.n) bins.push_back(b);
+  auto collect = [&](bool team, int k, bool m_tm) {
+    ClusterBin b{(int)list.size(), 0, team ? cl_team_of(k) : cl_size_of(k), 0, 0, m_tm, team};
+    for (int s = 0; s < n_sys; ++s) {
+      if (choice[s].size != k || choice[s].m_tm != m_tm || choice[s].team != team) continue;
+      const ClusterShare& sh = team ? model(s)->cl_team[k] : model(s)->cl_share[k];
+      // all of a CTA's K resident where it fits, else whatever room is left
+      const size_t all = m_tm ? dev->smem
+                              : cluster_smem_bytes(sh, precond, false, team) +
+                                    (size_t)CL_POS_BYTES * (sh.positions + 2);
+      b.smem = std::max(b.smem, (int)std::min((size_t)dev->smem, all));
+      b.threads = std::max(b.threads, 32 * cluster_warps(sh.own_tiles));
+      list.push_back(s);
+      ++b.n;
     }
+    if (b.n) bins.push_back(b);
+  };
+  for (int m_tm = 0; m_tm < 2; ++m_tm) {
+    for (int k = 0; k < CL_TEAMS; ++k) collect(true, k, m_tm);
+    for (int k = CL_SIZES - 1; k >= 0; --k) collect(false, k, m_tm);
+  }
   *fits = !list.empty();
   return SSO_OK;
 }
 
-// One round: up to max_steps CG steps of every system of the bins, each bin
-// on a stream of its own, joined back to B's stream.
+// One round: up to max_steps CG steps of every system of the bins, each bin of
+// clusters on a stream of its own, joined back to B's stream.  Teams' launches
+// follow one another (each fills the device), after the clusters.
 sso_status launch_bins(sso_batch* B, const std::vector<ClusterBin>& bins, const int* d_list,
                        int precond, int max_steps) {
-  const int nb = (int)bins.size();
-  if (nb > 1) {
+  auto launch = [&](const ClusterBin& b, int first, int n, cudaStream_t s) {
+    CL(launch_cluster_cg(B->d_sys, d_list + first, n, b.size, b.threads, b.smem, precond, b.m_tm,
+                         b.team, B->d_slots, B->d_n_active, max_steps, s),
+       1);
+    return SSO_OK;
+  };
+  int nc = 0;  // bins of clusters
+  for (const ClusterBin& b : bins) nc += !b.team;
+  if (nc > 1) {
     if (!B->cl_fork) CK(cudaEventCreateWithFlags(&B->cl_fork, cudaEventDisableTiming));
-    for (int k = 0; k < nb - 1; ++k) {
+    for (int k = 0; k < nc - 1; ++k) {
       if (!B->cl_stream[k])
         CK(cudaStreamCreateWithFlags(&B->cl_stream[k], cudaStreamNonBlocking));
       if (!B->cl_join[k]) CK(cudaEventCreateWithFlags(&B->cl_join[k], cudaEventDisableTiming));
     }
     CK(cudaEventRecord(B->cl_fork, B->stream));
   }
-  for (int k = 0; k < nb; ++k) {
-    const ClusterBin& b = bins[k];
+  int k = 0;
+  for (const ClusterBin& b : bins) {
+    if (b.team) continue;
     cudaStream_t s = k == 0 ? B->stream : B->cl_stream[k - 1];
     if (k > 0) CK(cudaStreamWaitEvent(s, B->cl_fork, 0));
-    CL(launch_cluster_cg(B->d_sys, d_list + b.first, b.n, b.size, b.threads, b.smem, precond,
-                         b.m_tm, B->d_n_active, max_steps, s),
-       1);
+    const sso_status st = launch(b, b.first, b.n, s);
+    if (st != SSO_OK) return st;
     if (k > 0) {
       CK(cudaEventRecord(B->cl_join[k - 1], s));
       CK(cudaStreamWaitEvent(B->stream, B->cl_join[k - 1], 0));
     }
+    ++k;
+  }
+  if (nc == (int)bins.size()) return SSO_OK;
+  const ClusterDevice* dev = nullptr;
+  const sso_status st = cluster_device(&dev);
+  if (st != SSO_OK) return st;
+  for (const ClusterBin& b : bins) {
+    if (!b.team) continue;
+    const int per = std::min(dev->ctas / b.size, CL_MAX_TEAMS);
+    for (int at = 0; at < b.n; at += per) {
+      const sso_status ls = launch(b, b.first + at, std::min(per, b.n - at), B->stream);
+      if (ls != SSO_OK) return ls;
+    }
   }
   return SSO_OK;
 }
+
+// The CTAs of a team wait for one another, so that all of them must come to
+// run: one batch at a time has teams on the device (held from a launch until
+// its completion; other kernels beside them end by themselves).
+std::mutex g_team_mutex;
 
 // CG steps of a system per launch: long enough that loading a system (some
 // microseconds) does not count, short enough that the host sees finished
@@ -1230,7 +1274,7 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
   bool cluster = false;
   std::vector<ClusterBin> bins;
   if (o->precision == SSO_FP32_IR && !B->profiling) {
-    sso_status st = plan_bins(B->n_sys, active, o->precond, 1,
+    sso_status st = plan_bins(B->n_sys, active, o->precond, 1, true,
                               [B](int s) { return B->models[s]; }, B->h_list, bins, &cluster);
     if (st != SSO_OK) return st;
   }
@@ -1297,7 +1341,11 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
     const int steps = o->timeout_ms > 0.0 ? std::min(kClusterSteps, o->iters_per_launch)
                                           : kClusterSteps;
     const long long max_launches = (2LL * o->max_iter + 4LL * o->max_sweeps) / steps + 8;
+    const bool teams = std::any_of(bins.begin(), bins.end(),
+                                   [](const ClusterBin& b) { return b.team; });
     for (long long launches = 1;; ++launches) {
+      std::unique_lock<std::mutex> lock(g_team_mutex, std::defer_lock);
+      if (teams) lock.lock();
       sso_status st = launch_bins(B, bins, B->d_list, o->precond, steps);
       if (st != SSO_OK) return st;
       CK(cudaMemcpyAsync(B->h_flag + 2, B->d_n_active, 2 * sizeof(int), cudaMemcpyDeviceToHost,
@@ -1522,8 +1570,7 @@ void plan_cluster(sso_model* M, const HostTopo& T) {
   const size_t room = (size_t)std::max(M->n_eb, M->n_blocks) * 36 * sizeof(double);
   M->cluster_ok = n_chunks_of(M) <= CL_MAX_CHUNKS && cluster_pack_bytes(M) <= room;
   if (!M->cluster_ok) return;
-  for (int k = 0; k < CL_SIZES; ++k) {
-    const int C = cl_size_of(k);
+  auto share = [&](int C) {
     int win = 0, pos = 0;
     for (int r = 0; r < C; ++r) {  // the kernel's split of the tiles
       const int t0 = (int)((long long)M->n_tiles * r / C);
@@ -1537,14 +1584,16 @@ void plan_cluster(sso_model* M, const HostTopo& T) {
       if (hi > lo) win = std::max(win, hi - lo);
       pos = std::max(pos, T.toff[t1] - T.toff[t0]);
     }
-    int members = 0;
+    int members = 0;  // of the aggregates r, r + C, ...
     for (int r = 0; r < C; ++r) {
       int m = 0;
       for (int g = r; g < T.n_agg; g += C) m += T.agg_ptr[g + 1] - T.agg_ptr[g];
       members = std::max(members, m);
     }
-    M->cl_share[k] = {M->n_tiles, (M->n_tiles + C - 1) / C, win, pos, members};
-  }
+    return ClusterShare{M->n_tiles, (M->n_tiles + C - 1) / C, win, pos, members};
+  };
+  for (int k = 0; k < CL_SIZES; ++k) M->cl_share[k] = share(cl_size_of(k));
+  for (int k = 0; k < CL_TEAMS; ++k) M->cl_team[k] = share(cl_team_of(k));
 }
 
 // Host half of a model: the mesh, validated, and its scatter map, node
@@ -2202,6 +2251,7 @@ sso_status create_batch(sso_model* const* models, int32_t n, sso_batch** out, bo
   c.take<int>(2);
   c.take<SetupJob>(n);
   c.take<int>(n);
+  c.take<unsigned long long>(CL_SLOT_BYTES / 8);
   const size_t bytes = align_up(c.off, 256);
   std::vector<SetupJob> jobs(n);
   for (int s = 0; s < n; ++s) {
@@ -2229,6 +2279,7 @@ sso_status create_batch(sso_model* const* models, int32_t n, sso_batch** out, bo
   B->d_ccount = d.take<int>(2);
   B->d_jobs = d.take<SetupJob>(n);
   B->d_list = d.take<int>(n);
+  B->d_slots = d.take<unsigned long long>(CL_SLOT_BYTES / 8);
   B->grid_restrict = (B->n_aggs + 7) / 8;  // one warp per (system, aggregate)
   B->grid_csolve = n * COARSE_ROW_BLOCKS;  // one CTA per work item
   const int ccount[2] = {B->n_aggs, n};
@@ -2922,7 +2973,7 @@ sso_status server_upload_tables(sso_server* S, std::vector<std::vector<TileDesc>
     std::vector<char> active(S->max_sys, 0);
     for (int slot : S->running) active[slot] = 1;
     bool fits = false;
-    sso_status st = plan_bins(S->max_sys, active, S->opts.precond, S->lane_count,
+    sso_status st = plan_bins(S->max_sys, active, S->opts.precond, S->lane_count, false,
                               [S](int slot) { return S->slot_req[slot]->M; }, B->h_list,
                               S->bins, &fits);
     if (st != SSO_OK) return st;

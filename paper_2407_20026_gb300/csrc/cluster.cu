@@ -1,4 +1,5 @@
-// Batched FP32 CG with FP64 refinement, one thread-block cluster per system.
+// Batched FP32 CG with FP64 refinement, one thread-block cluster per system, or
+// one team of CTAs over a whole, a half or a quarter of the chip.
 //
 // What bounds it: the latency of an iteration.  The two-kernel engine (pcg.cu)
 // streams every system's K from HBM in every iteration and pays two launches'
@@ -12,6 +13,15 @@
 // one system 16.1 -> 7.0 us an iteration (208.8 -> 90.2 ms a solve; on 16 SMs),
 // 48 systems 1.58 -> 0.71 us a system-iteration (945 -> 424 ms); two-level
 // preconditioner, one 28.8 -> 14.2 us, 128 systems 403 -> 256 ms.
+//
+// Larger systems (and a few middle-sized ones together) take teams of 152, 76
+// or 38 CTAs of a cooperative launch: more room for K on chip and more SMs to
+// stream the rest, but z goes through global memory and the barriers too
+// (team_sync: 4,000 to 6,000 clocks an iteration more than a cluster's).
+// Measured, us an iteration, two-kernel engine -> team: 256 x 256 shell
+// (396,294 DOF, K 85 MB, 57 MB of it streamed) 36 -> 13.6, 128 x 128 shell
+// 28 -> 8.7, 100 x 100 grid shell 25 -> 8.0 (on a cluster of 16: 13.8).  The
+// coarse correction needs a cluster: two-level systems do not take teams.
 //
 // The arithmetic is the two-kernel engine's, so every result is the same bits
 // and the two engines can follow one another on a system at any step:
@@ -255,6 +265,14 @@ struct ClShared {
   Apx rz;
   double ex_pq, ex_rz, ex_rr;  // exact_sums
   double red[2 * CL_MAX_VWARPS];
+  // teams without a cluster: the next barrier's set of words, whether a barrier
+  // gave up, the words and their last values, the warps' sums and the team's
+  unsigned epoch;
+  int lost, team, copy;
+  unsigned long long *slots, before[2][6];
+  int* flags;
+  unsigned long long words[CL_MAX_THREADS / 32][6];
+  Fix tot[2];
 };
 
 // finite / positive and finite, by the bits (FP64 compares cost 64 clocks)
@@ -274,9 +292,12 @@ __device__ __forceinline__ bool f64_positive(double x) {
 // (a double-float) is instead rounded to a 64-bit integer on a grid of 2^-50
 // of the previous iteration's sum; the integers are added exactly, in any
 // order, and the quotient is formed to about 2^-41 with a bound on everything
-// that separates it from the FP64 result: the grid (2^-49 of the sum per
-// partial and part), the rounding of the FP64 chains (at most 20 2^-53 of
-// the sum of magnitudes, which may be 2^10 times the sum), the quotient's own.
+// that separates it from the FP64 result: the grid (at most 1.25 2^-49 of the
+// sum per partial: a high part is truncated only where the low part is less
+// than a quarter of the grid; 2^-34.5 for p^T q's 18,432 partials of twelve
+// chunks, 2^-37.1 for r^T z), the rounding of the FP64 chains (at most 24 2^-53
+// of the sum of magnitudes, which may be 2^10 times the sum), the quotient's
+// own: 0.93 2^-34 together.
 // When a float's rounding (or the comparison) is the same anywhere within
 // 2^-34, it is the two-kernel engine's; else, and where a sum leaves the
 // grid's range, the exact sums are formed (exact_sums), about once in 300
@@ -330,6 +351,103 @@ __device__ __noinline__ Fix fix_total(const Fix* slot, int n, int lane) {
     }
   }
   return fix_warp_sum(t);
+}
+
+// ---------------------------------------------------------------------------
+// The barrier of a team of CTAs that is not a cluster (a cooperative launch's,
+// all resident at once), with up to two sums over the warps of all CTAs: every
+// warp calls team_add for each, then all call team_sync, which leaves them in
+// sh.tot.  A sum goes as three words of integers, which add up in any order.
+// Each CTA adds its six words, with 1 in the upper 16 bits, to each of
+// CL_TEAM_COPIES lines, and polls one of these (a line that all SMs poll serves
+// late adds late, and its readers unevenly).  Words are never reset: a word's
+// growth since the last barrier of its set is the team's sum once it holds the
+// team's count, so that a sum costs no round trip beyond the barrier's own.
+// Two sets alternate, as a CTA may be one barrier ahead of a slow reader.
+// data: global stores before are visible to the team after (else only the sums
+// are).  Measured in a loop of barriers alone, 152 CTAs: one counter 2,000
+// clocks (3,000 with data's fences), this 1,800 to 2,200; a slot per CTA that
+// all poll 6,200, a mailbox per CTA that all store into 4,700, clusters of 4
+// and their mailboxes 3,700.  256 x 256 shell, us an iteration: slots 21,
+// mailboxes 15.9, this 13.6.
+// A CTA that waits for some seconds gives up: it sets the error flag, and its
+// later barriers do not wait.
+constexpr long long kTeamWait = 8000000000ll;  // clocks
+constexpr int kTeamBias = 1 << 24;             // keeps the upper halves positive
+
+// The warp's share of sum k (one lane).
+__device__ __forceinline__ void team_add(ClShared& sh, int k, Fix f) {
+  if (f.s >= (1ll << 55) || f.s <= -(1ll << 55)) f = Fix{0, f.a, 1u};
+  unsigned long long* w = sh.words[threadIdx.x >> 5] + 3 * k;
+  w[0] = (unsigned)f.s;
+  w[1] = (unsigned long long)((f.s >> 32) + kTeamBias);
+  w[2] = ((unsigned long long)f.bad << 34) | f.a;
+}
+__device__ __forceinline__ void fence_gpu() {
+  asm volatile("fence.acq_rel.gpu;" ::: "memory");
+}
+__device__ __noinline__ void team_sync(ClShared& sh, bool data) {
+  const int lane = threadIdx.x & 31;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const int W = blockDim.x >> 5, word = lane % 6, part = lane / 6;
+    unsigned long long v = 0ull;
+    if (lane < 30)
+#pragma unroll 1
+      for (int w = part; w < W; w += 5) v += sh.words[w][word];
+    unsigned long long add = 1ull << 48;
+#pragma unroll
+    for (int p = 0; p < 5; ++p) add += __shfl_sync(0xffffffffu, v, word + 6 * p);
+    const unsigned set = sh.epoch;
+    unsigned long long* line = sh.slots + 16 * CL_TEAM_COPIES * set;
+    if (data) fence_gpu();
+    if (lane < 30) {
+#pragma unroll
+      for (int c = 0; c < CL_TEAM_COPIES; c += 5)
+        asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(line + 16 * (c + part) +
+                                                                      word),
+                     "l"(add)
+                     : "memory");
+    }
+    // the first six lanes' words (the others read them too)
+    const unsigned long long* p = line + 16 * sh.copy + word;
+    const unsigned long long before = sh.before[set][word];
+    const long long t0 = clock64();
+    unsigned long long now;
+    bool wait;
+    do {
+      asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(now) : "l"(p) : "memory");
+      wait = __any_sync(0xffffffffu, (int)((now - before) >> 48) != sh.team);
+      if (wait && (sh.lost || clock64() - t0 > kTeamWait)) {
+        wait = false;
+        __syncwarp();
+        if (lane == 0) {
+          sh.lost = 1;
+          atomicExch(sh.flags + 1, 1);
+        }
+      }
+      wait = __any_sync(0xffffffffu, wait);
+    } while (wait);
+    if (data) fence_gpu();
+    if (lane < 6) sh.before[set][word] = now;
+    now = (now - before) & ((1ull << 48) - 1ull);
+    const unsigned long long hi = __shfl_down_sync(0xffffffffu, now, 1);
+    const unsigned long long ab = __shfl_down_sync(0xffffffffu, now, 2);
+    if (lane == 0 || lane == 3)
+      sh.tot[lane / 3] =
+          Fix{(long long)now + (((long long)hi - (long long)sh.team * W * kTeamBias) << 32),
+              (unsigned)ab, (unsigned)(ab >> 34)};
+    if (lane == 0) sh.epoch = set ^ 1u;
+  }
+  __syncthreads();
+}
+// Barrier after global stores that the other CTAs read.
+template <bool GRID>
+__device__ __forceinline__ void all_sync(ClShared& sh) {
+  if (GRID)
+    team_sync(sh, true);
+  else
+    cl_sync();
 }
 
 __device__ __forceinline__ Apx apx_bits(unsigned long long m, int e) {  // m: bit 63 set
@@ -398,11 +516,12 @@ __device__ __noinline__ double vwarp_sum(const double* buf, int v, int n, int la
 
 // Sum of the chunk sums x[0 .. n) by one thread: the tree of a warp.
 __device__ __noinline__ double chunk_tree(const double* x, int n) {
-  double t[CL_MAX_CHUNKS];
+  double t[16];
+  static_assert(CL_MAX_CHUNKS <= 16, "");
 #pragma unroll
-  for (int k = 0; k < CL_MAX_CHUNKS; ++k) t[k] = k < n ? x[k] : 0.0;
+  for (int k = 0; k < 16; ++k) t[k] = k < n ? x[k] : 0.0;
 #pragma unroll
-  for (int o = CL_MAX_CHUNKS / 2; o > 0; o >>= 1)
+  for (int o = 8; o > 0; o >>= 1)
 #pragma unroll
     for (int k = 0; k < o; ++k) t[k] += t[k + o];
   return t[0];
@@ -457,7 +576,7 @@ __device__ __noinline__ double coarse_dot(const float* y, const float* w, int nc
 // The FP64 sums themselves, by every CTA from all partials (through global
 // memory): r^T z and r^T r of
 // the iteration in buffer `par` (ex_rz, ex_rr) and, with_a, p^T q (ex_pq).
-template <bool TWO>
+template <bool TWO, bool GRID>
 __device__ __noinline__ void exact_sums(ClShared& sh, int par, bool with_a) {
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, W = blockDim.x >> 5;
   const int n_tiles = sh.sys.n_tiles, n_ow = sh.n_ow, n_chunks = sh.sys.n_chunks;
@@ -478,7 +597,7 @@ __device__ __noinline__ void exact_sums(ClShared& sh, int par, bool with_a) {
       bufA[WARPS * sh.T0 + g] = df_to_f64(DF{v.x, v.y});
     }
   }
-  cl_sync();
+  all_sync<GRID>(sh);
   if (w < 2) {
     const double s = total_b(bufB + (size_t)w * n_tiles, n_tiles, n_chunks, lane,
                              sh.red + CL_MAX_VWARPS + CL_MAX_CHUNKS * w);
@@ -623,18 +742,20 @@ __device__ __noinline__ void sweep_scalars(ClShared& sh, int state, double s1, d
 
 // A system's CG on one cluster, up to max_steps steps (an A and a B phase
 // each) from the state in its SysScalars, which it leaves ready for more.
-template <bool TWO, bool JAC, int KREG>
+template <bool TWO, bool JAC, int KREG, bool GRID>
 __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) cluster_cg_kernel(
     const SysDesc* __restrict__ sys, const int* __restrict__ list, int* __restrict__ flags,
-    int max_steps, int smem_bytes, int tm_cols, int m_tm) {
+    int max_steps, int smem_bytes, int tm_cols, int m_tm, int team, unsigned long long* slots) {
   extern __shared__ __align__(16) unsigned char cl_smem[];
   __shared__ ClShared sh;
-  const unsigned rank = cl_rank(), C = cl_size();
+  static_assert(!(TWO && GRID), "the coarse correction exchanges through a cluster");
+  const unsigned C = GRID ? (unsigned)team : cl_size();
+  const unsigned rank = GRID ? blockIdx.x % C : cl_rank();
   const int tid = threadIdx.x, nth = blockDim.x, w = tid >> 5, lane = tid & 31;
   {
     const SysDesc& G = sys[list[blockIdx.x / C]];
     if (*(volatile const int*)&G.sc->state == ST_DONE) return;  // alike in every CTA
-    cl_arrive();  // waited for before the first store to another CTA
+    if (!GRID) cl_arrive();  // waited for before the first store to another CTA
 #pragma unroll 1
     for (int i = tid; i < (int)(sizeof(SysDesc) / 4); i += nth)
       reinterpret_cast<int*>(&sh.sys)[i] = reinterpret_cast<const int*>(&G)[i];
@@ -646,7 +767,17 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
     sh.n_done = 1;
     sh.lo = INT_MAX;
     sh.hi = 0;
+    if (GRID) {
+      sh.epoch = 0u;
+      sh.lost = 0;
+      sh.team = team;
+      sh.copy = (int)rank % CL_TEAM_COPIES;
+      sh.slots = slots + CL_TEAM_WORDS * (blockIdx.x / C);
+      sh.flags = flags;
+    }
   }
+  if (GRID && tid < 12) sh.before[tid / 6][tid % 6] = 0ull;
+  if (GRID && lane < 6) sh.words[w][lane] = 0ull;
   __syncthreads();
   const SysDesc& S = sh.sys;
   const int n = S.n_nodes, n_tiles = S.n_tiles, n_ow = WARPS * n_tiles;
@@ -680,14 +811,14 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
     return p;
   };
   // first what other CTAs store into, at the same place in each
-  Fix* fixA = reinterpret_cast<Fix*>(take(16 * (size_t)n_tiles));  // p^T q per tile
-  Fix* fixB = reinterpret_cast<Fix*>(take(16 * (size_t)n_tiles));  // r^T z per tile
-  Fix* fixR = reinterpret_cast<Fix*>(take(16 * (size_t)n_tiles));  // r^T r per tile
+  Fix* fixA = reinterpret_cast<Fix*>(take(GRID ? 0 : 16 * (size_t)n_tiles));  // p^T q per tile
+  Fix* fixB = reinterpret_cast<Fix*>(take(GRID ? 0 : 16 * (size_t)n_tiles));  // r^T z per tile
+  Fix* fixR = reinterpret_cast<Fix*>(take(GRID ? 0 : 16 * (size_t)n_tiles));  // r^T r per tile
   Fix* fixC = reinterpret_cast<Fix*>(take(TWO ? 16 * 8 * COARSE_ROW_BLOCKS : 0));  // w^T y
   float* wS = reinterpret_cast<float*>(take(TWO ? 8 * COARSE_MAX_N : 0));  // two iterations
   float* yS = reinterpret_cast<float*>(take(TWO ? 8 * COARSE_MAX_N : 0));
   int* aptr = reinterpret_cast<int*>(take(TWO ? 4 * (COARSE_MAX_AGG + 1) : 0));
-  float* Zw = reinterpret_cast<float*>(take(24 * (size_t)wn));  // z (two-level: z_b) of the window
+  float* Zw = reinterpret_cast<float*>(take(GRID ? 0 : 24 * (size_t)wn));  // z (two-level: z_b) of the window
   float* P = reinterpret_cast<float*>(take(24 * (size_t)wn));
   float* Q = reinterpret_cast<float*>(take(24 * (size_t)nown));
   float* R = reinterpret_cast<float*>(take(24 * (size_t)nown));
@@ -873,9 +1004,10 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
 #pragma unroll 1
     for (int i = tid; i < 3 * wn; i += nth) {
       reinterpret_cast<float2*>(P)[i] = __ldcg(p2 + i);
-      reinterpret_cast<float2*>(Zw)[i] = __ldcg(z2 + i);
+      if (!GRID) reinterpret_cast<float2*>(Zw)[i] = __ldcg(z2 + i);
     }
   }
+  bool z_alt = false;   // teams without a cluster: z is in S.zb, not S.z
   bool zdirect = true;  // Zw holds z itself (two-level: until this launch's first z_b)
   int state = sh.sc.state, parity = sh.sc.parity, iters = sh.sc.iters, inner = sh.sc.inner;
   // scalars of the iteration, alike in every thread: r^T z (exact while known),
@@ -888,25 +1020,43 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
   // Every CTA has started by now (one that has not must not be stored to: the
   // CTAs of a cluster are placed together, but an SM that has to drain another
   // kernel first starts its own late) ...
-  cl_wait();
-  if (tid < (int)C) {
+  if (!GRID) cl_wait();
+  if (!GRID && tid < (int)C) {
     cl_st(cl_map(smem_addr(&sh.wlo[rank]), tid), lo);
     cl_st(cl_map(smem_addr(&sh.whi[rank]), tid), lo + wn);
   }
-  cl_sync();  // ... and has read the system's state and set up its windows
+  if (!GRID) cl_sync();  // ... and has read the system's state and set up its windows
   unsigned dest = 0u;  // CTAs whose windows reach this warp's nodes
 #pragma unroll 1
-  for (unsigned c = 0; c < C; ++c)
+  for (unsigned c = 0; !GRID && c < C; ++c)
     if (sh.wlo[c] < min(n, TILE * tb) && sh.whi[c] > TILE * ta && tb > ta) dest |= 1u << c;
 
   int products = 0;  // matrix products of this launch
 #pragma unroll 1
-  for (int step = 0; step < max_steps && state != ST_DONE; ++step) {
+  for (int step = 0; step < max_steps && state != ST_DONE && !(GRID && sh.lost); ++step) {
     float alpha = 0.f;
     // ------------------------------------------------------------- phase A
     if (state == ST_PCG) {
       const bool first = inner == 0;
-      if (!TWO || zdirect) {
+      if (GRID) {
+        const float b = first ? 0.f : beta;
+        float2* P2 = reinterpret_cast<float2*>(P);
+        const float2* Z2 = reinterpret_cast<const float2*>((const float*)(z_alt ? S.zb : S.z) +
+                                                           6 * (size_t)lo);
+#pragma unroll 1
+        for (int i = tid; i < 3 * wn; i += 4 * nth) {
+          float2 z[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (i + u * nth < 3 * wn) z[u] = __ldcg(Z2 + i + u * nth);
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (i + u * nth < 3 * wn) {
+              const float2 p = first ? z[u] : P2[i + u * nth];
+              P2[i + u * nth] = make_float2(fmaf(b, p.x, z[u].x), fmaf(b, p.y, z[u].y));
+            }
+        }
+      } else if (!TWO || zdirect) {
         const float b = first ? 0.f : beta;
         float2* P2 = reinterpret_cast<float2*>(P);
         const float2* Z2 = reinterpret_cast<const float2*>(Zw);
@@ -1015,6 +1165,7 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
       // levels 16, 8 and 4 of the tree over the rows l = j mod 4 of the group's
       // 30 (lanes 30 and 31 of that tree hold zero), two shuffles the last two
       __syncwarp();
+      Fix pq_sum{0, 0u, 0u};
 #pragma unroll 1
       for (int t = ta; t < tb; ++t) {
         const int g = WARPS * t + (lane >> 2), j = lane & 3;
@@ -1045,17 +1196,27 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
           sh.gA[g - WARPS * T0] = make_float2(v.hi, v.lo);
           f = to_fix(v, kA);
         }
-        f = fix_warp_sum(f);
-        if (lane < (int)C) push_fix(sh.fixA + t, f, lane);
+        if (GRID) {
+          pq_sum = Fix{pq_sum.s + f.s, pq_sum.a + f.a, pq_sum.bad | f.bad};
+        } else {
+          f = fix_warp_sum(f);
+          if (lane < (int)C) push_fix(sh.fixA + t, f, lane);
+        }
       }
-      cl_sync();
+      if (GRID) {
+        pq_sum = fix_warp_sum(pq_sum);
+        if (lane == 0) team_add(sh, 0, pq_sum);
+        team_sync(sh, false);
+      } else {
+        cl_sync();
+      }
       // alpha = r^T z / p^T q, by every warp
       Apx pq;
-      const Fix fa = fix_total(sh.fixA, S.n_tiles, lane);
+      const Fix fa = GRID ? sh.tot[0] : fix_total(sh.fixA, S.n_tiles, lane);
       if (have_kA && apx_fix(fa, kA, pq) && apx_quotient(rz, pq, alpha)) {
         kA = kGrid - pq.e;
       } else {
-        exact_sums<TWO>(sh, par, true);
+        exact_sums<TWO, GRID>(sh, par, true);
         const double s = sh.ex_pq;
         if (!f64_positive(s)) {
           if (tid == 0) sh.sc.status = SSO_ERR_SINGULAR;
@@ -1070,7 +1231,7 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
     } else if (state != ST_FOLD) {  // INIT, RESID
       const int n_ow = sh.n_ow, n_vw = (n_ow + 255) / 256;
       residual_phase(S, state, WARPS * T0, WARPS * T1, n1, n_ow);
-      cl_sync();
+      all_sync<GRID>(sh);
 #pragma unroll 1
       for (int v = w; v < 2 * n_vw; v += nth >> 5) {
         const bool second = v >= n_vw;
@@ -1092,7 +1253,7 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
         D[i] = 0.f;
       }
       state = ST_RESID;
-      cl_sync();  // the other CTAs read x next
+      all_sync<GRID>(sh);  // the other CTAs read x next
       continue;
     }
     if (state != ST_PCG) {
@@ -1108,6 +1269,9 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
       scale_residual(S, rr64, n0, nown, R);
     }
     par ^= 1;
+    // z goes to the buffer that no CTA still reads
+    float* zn = GRID ? (float*)(z_alt ? S.z : S.zb) : nullptr;
+    Fix b_sum{0, 0u, 0u};
     __syncwarp();
 #pragma unroll 1
     for (int t = ta; t < tb; ++t) {
@@ -1173,6 +1337,7 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
           cl_st2(a + 16, zv[4], zv[5]);
         }
       }
+      if (GRID && lane < TILE && node < n1) sts6(zn + 6 * (size_t)node, zv);
       if (lane < TILE && node < n1) {
         d1 = df_prod(rv[0], zv[0]);
         d2 = df_prod(rv[0], rv[0]);
@@ -1199,9 +1364,16 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
       v.hi = __shfl_sync(0xffffffffu, v.hi, lane & 16);
       v.lo = __shfl_sync(0xffffffffu, v.lo, lane & 16);
       const Fix f = to_fix(v, lane < 16 ? kB : kR);
-      if ((lane & 15) < (int)C) push_fix((lane < 16 ? sh.fixB : sh.fixR) + t, f, lane & 15);
+      if (GRID)
+        b_sum = Fix{b_sum.s + f.s, b_sum.a + f.a, b_sum.bad | f.bad};
+      else if ((lane & 15) < (int)C)
+        push_fix((lane < 16 ? sh.fixB : sh.fixR) + t, f, lane & 15);
     }
-    cl_sync();
+    if (GRID) {
+      if ((lane & 15) == 0) team_add(sh, lane >> 4, b_sum);
+      z_alt = !z_alt;
+    }
+    all_sync<GRID>(sh);
     if (TWO) {
       // coarse correction: w = P^T r, y = A_c^-1 w, r^T z = r^T z_b + w^T y
       const int nc = 6 * S.n_agg;
@@ -1292,7 +1464,7 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
       ++iters;
       ++inner;
       if (w == 0) {
-        Fix f = fix_total(sh.fixB, S.n_tiles, lane);
+        Fix f = GRID ? sh.tot[0] : fix_total(sh.fixB, S.n_tiles, lane);
         if (TWO) {
           const int n_rb = (6 * S.n_agg + COARSE_ROWS_PER_BLOCK - 1) / COARSE_ROWS_PER_BLOCK;
           const Fix g = fix_total(sh.fixC, 8 * n_rb, lane);
@@ -1308,7 +1480,7 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
         }
       }
       if (w == 1) {
-        const Fix f = fix_total(sh.fixR, S.n_tiles, lane);
+        const Fix f = GRID ? sh.tot[1] : fix_total(sh.fixR, S.n_tiles, lane);
         Apx rr{1.f, 0.f, 0};
         bool clear;
         const bool end = fix_le(f, kR, sh.thr, clear);
@@ -1329,10 +1501,10 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
       } else {
         double rz_old = sh.rz_known;
         if (!known) {
-          exact_sums<TWO>(sh, par ^ 1, false);
+          exact_sums<TWO, GRID>(sh, par ^ 1, false);
           rz_old = sh.ex_rz;
         }
-        exact_sums<TWO>(sh, par, false);
+        exact_sums<TWO, GRID>(sh, par, false);
         const double s1 = sh.ex_rz, s2 = sh.ex_rr;
         if (!(f64_finite(s1) && f64_finite(s2))) {
           if (tid == 0) sh.sc.status = SSO_ERR_SINGULAR;
@@ -1352,7 +1524,7 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
       kR = kGrid - e_rr;
       if (end || iters >= sh.sc.max_iter) state = ST_FOLD;
     } else {
-      exact_sums<TWO>(sh, par, false);
+      exact_sums<TWO, GRID>(sh, par, false);
       if (tid == 0) {
         sh.sc.iters = iters;
         sweep_scalars(sh, state, sh.ex_rz, sh.ex_rr);
@@ -1375,8 +1547,9 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
   }
   // leave the system as the two-kernel engine would: r, dx, p and z in global
   // memory, the scalars written by one thread
-  if (state == ST_PCG && !known) exact_sums<TWO>(sh, par, false);
-  if (state != ST_DONE) {
+  if (state == ST_PCG && !known) exact_sums<TWO, GRID>(sh, par, false);
+  const bool lost = GRID && sh.lost;  // a barrier gave up: the run has failed
+  if (state != ST_DONE && !lost) {
     float2* r2 = reinterpret_cast<float2*>((float*)S.r + 6 * (size_t)n0);
     float2* d2 = reinterpret_cast<float2*>((float*)S.dx + 6 * (size_t)n0);
     float2* p2 = reinterpret_cast<float2*>((float*)(parity ? S.p1 : S.p0) + 6 * (size_t)n0);
@@ -1387,7 +1560,13 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
       p2[i] = reinterpret_cast<const float2*>(P + 6 * (n0 - lo))[i];
     }
 #pragma unroll 1
-    for (int i = n0 + tid; i < n1; i += nth) {
+    for (int i = n0 + tid; GRID && z_alt && i < n1; i += nth) {
+      float z[6];
+      ldcg6((const float*)S.zb + 6 * (size_t)i, z);
+      sts6((float*)S.z + 6 * (size_t)i, z);
+    }
+#pragma unroll 1
+    for (int i = n0 + tid; !GRID && i < n1; i += nth) {
       float z[6];
       lds6(Zw + 6 * (i - lo), z);
       if (TWO && !zdirect) {
@@ -1405,8 +1584,8 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
     for (int k = 0; k < min(ns, cap); ++k)
       if (ring || products == 0) mbar_wait(bar + k, (rphase >> k) & 1u);
   if (tm_cols && w == 0) tm_free(sh.tmem, tm_cols);
-  cl_sync();  // no CTA leaves while another may still store into it
-  if (rank == 0 && tid == 0) {
+  if (!GRID) cl_sync();  // no CTA leaves while another may still store into it
+  if (rank == 0 && tid == 0 && !lost) {
     sh.sc.state = state;
     sh.sc.parity = parity;
     sh.sc.iters = iters;
@@ -1421,14 +1600,14 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
 }  // namespace
 
 // Shared memory of one CTA before resident K (the kernel carves the same sum).
-size_t cluster_smem_bytes(const ClusterShare& c, int precond, bool m_tm) {
+size_t cluster_smem_bytes(const ClusterShare& c, int precond, bool m_tm, bool team) {
   auto a = [](size_t b) { return (b + 15) & ~(size_t)15; };
   const size_t own = (size_t)TILE * c.own_tiles, nt = c.own_tiles;
-  size_t s = 3 * 16 * (size_t)c.n_tiles;
+  size_t s = team ? 0 : 3 * 16 * (size_t)c.n_tiles;
   if (precond == SSO_TWO_LEVEL)
     s += 16 * 8 * COARSE_ROW_BLOCKS + 2 * a(8 * COARSE_MAX_N) + a(4 * (COARSE_MAX_AGG + 1)) +
          16 * (size_t)c.window + 16 * (size_t)c.members;
-  s += 2 * a(24 * (size_t)c.window) + 3 * a(24 * own) + 8 * WARPS * nt + 32 * nt;
+  s += (team ? 1 : 2) * a(24 * (size_t)c.window) + 3 * a(24 * own) + 8 * WARPS * nt + 32 * nt;
   if (!m_tm) s += (precond == SSO_JACOBI ? 768 : 3072) * nt;
   s += 64 * (size_t)c.positions + a(4 * (nt + 1));
   return s + 8 * CL_MAX_RING * (CL_MAX_THREADS / 32) + 128;
@@ -1454,11 +1633,15 @@ static cudaError_t cluster_attributes(int* max_smem) {
   static int limit = 0;
   std::lock_guard<std::mutex> lock(mu);
   if (!limit) {
-    const void* fns[5] = {(const void*)cluster_cg_kernel<false, false, 0>,
-                          (const void*)cluster_cg_kernel<false, true, 0>,
-                          (const void*)cluster_cg_kernel<true, false, 0>,
-                          (const void*)cluster_cg_kernel<false, false, CL_KREG>,
-                          (const void*)cluster_cg_kernel<false, true, CL_KREG>};
+    const void* fns[9] = {(const void*)cluster_cg_kernel<false, false, 0, false>,
+                          (const void*)cluster_cg_kernel<false, true, 0, false>,
+                          (const void*)cluster_cg_kernel<true, false, 0, false>,
+                          (const void*)cluster_cg_kernel<false, false, CL_KREG, false>,
+                          (const void*)cluster_cg_kernel<false, true, CL_KREG, false>,
+                          (const void*)cluster_cg_kernel<false, false, 0, true>,
+                          (const void*)cluster_cg_kernel<false, true, 0, true>,
+                          (const void*)cluster_cg_kernel<false, false, CL_KREG, true>,
+                          (const void*)cluster_cg_kernel<false, true, CL_KREG, true>};
     int dev = 0, optin = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess)
@@ -1498,14 +1681,20 @@ static void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int
   cfg.numAttrs = 1;
 }
 
-cudaError_t cluster_limits(int* max_smem, int slots[CL_SIZES]) {
+cudaError_t cluster_limits(int* max_smem, int slots[CL_SIZES], int* max_ctas) {
   cudaError_t e = cluster_attributes(max_smem);
+  int dev = 0, coop = 0, sms = 0;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  *max_ctas = coop ? sms : 0;
   for (int k = 0; k < CL_SIZES && e == cudaSuccess; ++k) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[1];
     cluster_config(cfg, at, 1, cl_size_of(k), CL_MAX_THREADS, *max_smem, nullptr);
     slots[k] = 0;
-    e = cudaOccupancyMaxActiveClusters(&slots[k], cluster_cg_kernel<false, false, 0>, &cfg);
+    e = cudaOccupancyMaxActiveClusters(&slots[k], cluster_cg_kernel<false, false, 0, false>, &cfg);
   }
   return e;
 }
@@ -1521,8 +1710,9 @@ cudaError_t launch_cluster_pack(const SysDesc* sys, const int* list, int n_list,
 }
 
 cudaError_t launch_cluster_cg(const SysDesc* sys, const int* list, int n_list, int size,
-                              int threads, int smem, int precond, bool m_tm, int* flags,
-                              int max_steps, cudaStream_t s) {
+                              int threads, int smem, int precond, bool m_tm, bool team,
+                              unsigned long long* slots, int* flags, int max_steps,
+                              cudaStream_t s) {
   if (n_list <= 0) return cudaSuccess;
   int limit = 0;
   cudaError_t e = cluster_attributes(&limit);
@@ -1533,14 +1723,28 @@ cudaError_t launch_cluster_cg(const SysDesc* sys, const int* list, int n_list, i
   cluster_config(cfg, at, n_list, size, threads, smem, s);
   const int cols = cluster_tm_cols(smem);
   auto run = [&](auto kernel) {
-    return cudaLaunchKernelEx(&cfg, kernel, sys, list, flags, max_steps, smem, cols, (int)m_tm);
+    return cudaLaunchKernelEx(&cfg, kernel, sys, list, flags, max_steps, smem, cols, (int)m_tm,
+                              team ? size : 0, slots);
   };
-  if (precond == SSO_TWO_LEVEL) return run(cluster_cg_kernel<true, false, 0>);
+  if (team) {
+    if (precond == SSO_TWO_LEVEL || n_list > CL_MAX_TEAMS) return cudaErrorInvalidValue;
+    e = cudaMemsetAsync(slots, 0, CL_SLOT_BYTES, s);
+    if (e != cudaSuccess) return e;
+    at[0] = cudaLaunchAttribute{};
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    if (threads <= CL_REG_THREADS)
+      return precond == SSO_JACOBI ? run(cluster_cg_kernel<false, true, CL_KREG, true>)
+                                   : run(cluster_cg_kernel<false, false, CL_KREG, true>);
+    return precond == SSO_JACOBI ? run(cluster_cg_kernel<false, true, 0, true>)
+                                 : run(cluster_cg_kernel<false, false, 0, true>);
+  }
+  if (precond == SSO_TWO_LEVEL) return run(cluster_cg_kernel<true, false, 0, false>);
   if (threads <= CL_REG_THREADS)
-    return precond == SSO_JACOBI ? run(cluster_cg_kernel<false, true, CL_KREG>)
-                                 : run(cluster_cg_kernel<false, false, CL_KREG>);
-  return precond == SSO_JACOBI ? run(cluster_cg_kernel<false, true, 0>)
-                               : run(cluster_cg_kernel<false, false, 0>);
+    return precond == SSO_JACOBI ? run(cluster_cg_kernel<false, true, CL_KREG, false>)
+                                 : run(cluster_cg_kernel<false, false, CL_KREG, false>);
+  return precond == SSO_JACOBI ? run(cluster_cg_kernel<false, true, 0, false>)
+                               : run(cluster_cg_kernel<false, false, 0, false>);
 }
 
 }  // namespace sso

@@ -511,6 +511,16 @@ constexpr int cl_size_of(int k) {
   constexpr int size[CL_SIZES] = {1, 2, 3, 4, 6, 9, 16};
   return size[k];
 }
+// Teams of CTAs that are not clusters: all SMs, or a half or a quarter.
+constexpr int CL_TEAMS = 3;
+constexpr int cl_team_of(int k) {
+  constexpr int size[CL_TEAMS] = {152, 76, 38};
+  return size[k];
+}
+constexpr int CL_MAX_TEAMS = 4;  // of a launch
+// a team's barrier words: two sets of lines of 128 bytes
+constexpr int CL_TEAM_COPIES = 10, CL_TEAM_WORDS = 2 * CL_TEAM_COPIES * 16;
+constexpr size_t CL_SLOT_BYTES = 8 * (size_t)CL_TEAM_WORDS * CL_MAX_TEAMS;
 constexpr int CL_MAX_THREADS = 512;
 // Warps that own a CTA's tiles: as few rounds of tiles per warp as the limit
 // allows, evenly filled.
@@ -523,7 +533,7 @@ __host__ __device__ constexpr int cluster_warps(int own_tiles) {
 // positions of K of every warp there (not with the two-level preconditioner).
 constexpr int CL_REG_THREADS = 384, CL_KREG = 1;
 constexpr int CL_POS_BYTES = 36 * 4 * 32;  // a block position of a tile
-constexpr int CL_MAX_CHUNKS = 4;      // of CHUNK tiles: systems of up to 30,720 nodes
+constexpr int CL_MAX_CHUNKS = 12;     // of CHUNK tiles: up to 92,160 nodes (the sums' error bound)
 constexpr int CL_MAX_VWARPS = WARPS * CL_MAX_CHUNKS;
 // The largest share of a CTA: tiles of the system and of the CTA, nodes of
 // its window, block positions, members of its aggregates.
@@ -533,18 +543,19 @@ struct ClusterShare {
 // Shared memory of a CTA without resident K; block positions that each of
 // `warps` warps keeps in tensor memory in a CTA of `smem` bytes (-1: no room).
 // m_tm: the preconditioner is there too.
-size_t cluster_smem_bytes(const ClusterShare& c, int precond, bool m_tm);
+size_t cluster_smem_bytes(const ClusterShare& c, int precond, bool m_tm, bool team);
 int cluster_tm_positions(int smem, int own_tiles, int warps, bool m_tm);
 // The dynamic shared memory of a CTA and the clusters of each size that are
-// resident at once, with one CTA per SM.
-cudaError_t cluster_limits(int* max_smem, int slots[CL_SIZES]);
+// resident at once, with one CTA per SM; the CTAs of a cooperative launch.
+cudaError_t cluster_limits(int* max_smem, int slots[CL_SIZES], int* max_ctas);
 cudaError_t launch_cluster_pack(const SysDesc* sys, const int* list, int n_list, int max_nodes,
                                 cudaStream_t s);
 // Systems list[0 .. n_list), one cluster of `size` CTAs each, up to max_steps
 // CG steps; flags[0] is lowered by each system that finishes.
 cudaError_t launch_cluster_cg(const SysDesc* sys, const int* list, int n_list, int size,
-                              int threads, int smem, int precond, bool m_tm, int* flags,
-                              int max_steps, cudaStream_t s);
+                              int threads, int smem, int precond, bool m_tm, bool team,
+                              unsigned long long* slots, int* flags, int max_steps,
+                              cudaStream_t s);
 
 // Direct solve of a block-tridiagonal K by block cyclic reduction (chain.cu).
 // ws: chain_workspace_doubles(n) doubles; up[i]: index of block (i, i+1) in

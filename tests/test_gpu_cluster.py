@@ -154,3 +154,28 @@ def test_server_switches_engines(sso):
         assert got["stats"]["status"] == 0
         assert np.array_equal(got["u"], want["u"]) and got["C"] == want["C"]
     srv.close()
+
+
+@pytest.mark.parametrize("precond", ["jacobi", "block_jacobi"])
+@pytest.mark.parametrize("nodes", [30690, 30720, 30721, 92160, 92161])
+def test_teams_of_all_sms(sso, nodes, precond):
+    # systems beyond a cluster: 1,023 to 1,025 tiles (four and five reduction
+    # chunks), twelve chunks, and one node more, which takes the two kernels
+    _same(sso, [_strip(nodes)], precond=precond, rtol=1e-6, max_iter=200)
+
+
+@pytest.mark.parametrize("count", [2, 3, 5])
+def test_batches_of_teams(sso, count):
+    # several teams in a launch, several launches, and a cluster beside them
+    meshes = [meshgen.gridshell(110 + 9 * k, seed=k) for k in range(count)]
+    _same(sso, meshes + [meshgen.shell(9)], rtol=1e-6, max_iter=300)
+
+
+def test_teams_many_launches_and_adjoint(sso):
+    m = meshgen.shell(90, seed=2)
+    whole = _run(sso, [m], False, rtol=1e-6, max_iter=600)
+    cut = _run(sso, [m], False, rtol=1e-6, max_iter=600, timeout_ms=6e4, iters_per_launch=7)
+    assert cut[0][0]["iterations"] == whole[0][0]["iterations"]
+    assert np.array_equal(cut[1][0]["u"], whole[1][0]["u"])
+    g = np.random.default_rng(3).standard_normal(6 * m["xyz"].shape[0])
+    _same(sso, [m], g=[g], rtol=1e-6, max_iter=600)
