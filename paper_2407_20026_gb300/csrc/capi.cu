@@ -1108,8 +1108,7 @@ ClusterChoice cluster_choice(const sso_model* M, int n_sys, int precond, bool te
     const int slots = team ? std::min(d.ctas / C, CL_MAX_TEAMS) : d.slots[k], warps = cluster_warps(sh.own_tiles);
     if (slots < 1 || sh.window >= 65535 || (C > 1 && M->n_tiles < (team ? C : 2 * C))) return;
     // The preconditioner in shared memory, or in tensor memory (CTAs that use
-    // all of their shared memory anyway), whichever leaves less of K to L2; a
-    // position of K per warp in shared memory at least: the ring behind L2.
+    // all of their shared memory anyway), whichever leaves less of K to L2.
     // (In tensor memory a 100 x 100 grid shell, two-level, fits at all: 33.2 ->
     // 17.7 ms a solve; a 64 x 64 shell, two-level, 26.0 -> 25.7 ms.)
     const size_t share = (size_t)CL_POS_BYTES * sh.positions;
@@ -1118,8 +1117,7 @@ ClusterChoice cluster_choice(const sso_model* M, int n_sys, int precond, bool te
     for (int in_tm = 0; in_tm < (precond == SSO_JACOBI ? 1 : 2); ++in_tm) {
       const size_t need = cluster_smem_bytes(sh, precond, in_tm, team);
       const int pos = cluster_tm_positions(d.smem, sh.own_tiles, warps, in_tm);
-      if (pos < 0 || need + (size_t)CL_POS_BYTES * warps > (size_t)d.smem ||
-          (in_tm && need + share <= (size_t)d.smem))
+      if (pos < 0 || need > (size_t)d.smem || (in_tm && need + share <= (size_t)d.smem))
         continue;
       const size_t resident = d.smem - need + (size_t)CL_POS_BYTES * warps * pos;
       const size_t rest = share - std::min(share, resident);

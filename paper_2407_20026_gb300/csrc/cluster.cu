@@ -63,7 +63,6 @@ namespace {
 
 constexpr int CL_POS_F4 = 9 * 32;  // float4 per block position of a tile
 constexpr uint16_t kNoBlock = 0xffff;  // column slot past a row's end
-constexpr int CL_MAX_RING = 16;    // positions of a warp in shared memory
 
 // ---------------------------------------------------------------------------
 // Cluster primitives.
@@ -271,7 +270,7 @@ struct ClShared {
   int lost, team, copy;
   unsigned long long *slots, before[2][6];
   int* flags;
-  unsigned long long words[CL_MAX_THREADS / 32][6];
+  unsigned long long words[16][6];
   Fix tot[2];
 };
 
@@ -372,7 +371,7 @@ __device__ __noinline__ Fix fix_total(const Fix* slot, int n, int lane) {
 // mailboxes 15.9, this 13.6.
 // A CTA that waits for some seconds gives up: it sets the error flag, and its
 // later barriers do not wait.
-constexpr long long kTeamWait = 8000000000ll;  // clocks
+constexpr int kTeamPolls = 1 << 23;  // of about 700 clocks: some seconds
 constexpr int kTeamBias = 1 << 24;             // keeps the upper halves positive
 
 // The warp's share of sum k (one lane).
@@ -391,10 +390,10 @@ __device__ __noinline__ void team_sync(ClShared& sh, bool data) {
   __syncthreads();
   if (threadIdx.x < 32) {
     const int W = blockDim.x >> 5, word = lane % 6, part = lane / 6;
-    unsigned long long v = 0ull;
-    if (lane < 30)
-#pragma unroll 1
-      for (int w = part; w < W; w += 5) v += sh.words[w][word];
+    // (rows of warps that the CTA does not have are zero; no loops: the code
+    // comes from outer caches, and a branch stalls where it goes on)
+    const unsigned long long* mine = sh.words[part] + word;
+    const unsigned long long v = mine[0] + mine[5 * 6] + mine[10 * 6] + (part ? 0ull : mine[15 * 6]);
     unsigned long long add = 1ull << 48;
 #pragma unroll
     for (int p = 0; p < 5; ++p) add += __shfl_sync(0xffffffffu, v, word + 6 * p);
@@ -412,22 +411,15 @@ __device__ __noinline__ void team_sync(ClShared& sh, bool data) {
     // the first six lanes' words (the others read them too)
     const unsigned long long* p = line + 16 * sh.copy + word;
     const unsigned long long before = sh.before[set][word];
-    const long long t0 = clock64();
     unsigned long long now;
-    bool wait;
+    int polls = sh.lost ? 1 : kTeamPolls;
     do {
       asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(now) : "l"(p) : "memory");
-      wait = __any_sync(0xffffffffu, (int)((now - before) >> 48) != sh.team);
-      if (wait && (sh.lost || clock64() - t0 > kTeamWait)) {
-        wait = false;
-        __syncwarp();
-        if (lane == 0) {
-          sh.lost = 1;
-          atomicExch(sh.flags + 1, 1);
-        }
-      }
-      wait = __any_sync(0xffffffffu, wait);
-    } while (wait);
+    } while (!__all_sync(0xffffffffu, (int)((now - before) >> 48) == sh.team) && --polls);
+    if (polls == 0 && lane == 0) {
+      sh.lost = 1;
+      atomicExch(sh.flags + 1, 1);
+    }
     if (data) fence_gpu();
     if (lane < 6) sh.before[set][word] = now;
     now = (now - before) & ((1ull << 48) - 1ull);
@@ -777,7 +769,8 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
     }
   }
   if (GRID && tid < 12) sh.before[tid / 6][tid % 6] = 0ull;
-  if (GRID && lane < 6) sh.words[w][lane] = 0ull;
+  if (GRID)
+    for (int i = tid; i < 96; i += nth) sh.words[i / 6][i % 6] = 0ull;
   __syncthreads();
   const SysDesc& S = sh.sys;
   const int n = S.n_nodes, n_tiles = S.n_tiles, n_ow = WARPS * n_tiles;
@@ -850,13 +843,11 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
   float4* member = reinterpret_cast<float4*>(take(TWO ? 16 * (size_t)aptr[n_mine] : 0));
   uint16_t* slot = reinterpret_cast<uint16_t*>(take(64 * (size_t)(U1 - U0)));  // [position][lane]
   int* toffS = reinterpret_cast<int*>(take(4 * (size_t)(nt + 1)));
-  unsigned long long* bars =
-      reinterpret_cast<unsigned long long*>(take(8 * CL_MAX_RING * (size_t)W));
   sp = cl_smem + (((sp - cl_smem) + 127) & ~(size_t)127);
   ulonglong2* Kres = reinterpret_cast<ulonglong2*>(sp);
   const int left = smem_bytes - (int)(sp - cl_smem);
   // positions of K per warp in shared memory
-  const int cap = min(CL_MAX_RING, left > 0 ? left / (CL_POS_BYTES * W) : 0);
+  const int cap = left > 0 ? left / (CL_POS_BYTES * W) : 0;
   if (tid == 0) {
     sh.fixA = fixA;
     sh.fixB = fixB;
@@ -932,17 +923,14 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
   }
   // This warp's tiles are contiguous, so its K is one run of m positions: the
   // first nkr in registers (CTAs of few warps), the next ntm in tensor memory
-  // (the warp's share of its quadrant's columns), the ns others through its cap
-  // slots of shared memory (at least one: the plan's rule).  Where these do not
-  // all fit, the slots are a ring that bulk copies refill from L2: the k-th use
-  // of the ring is the k mod ns-th of them, in slot k mod cap, and a consumed
-  // slot takes the one cap uses on, so that the copies run ahead of the
-  // products, through the barriers and into the next iteration.
+  // (the warp's share of its quadrant's columns), the next ns in its share of
+  // shared memory, and the others come from L2 in every iteration, by plain
+  // loads that run three thirds of a position ahead of the products (the
+  // registers of a third are loaded again as soon as it has been used).  (A
+  // ring of slots in shared memory that bulk copies refill: XXX)
   const int ta = w < W ? T0 + nt * w / W : T1, tb = w < W ? T0 + nt * (w + 1) / W : T1;
   const int pa = __ldg(S.toff + ta), m = __ldg(S.toff + tb) - pa;
   if (tm_cols && w == 0) tm_alloc(&sh.tmem, tm_cols);
-  if (w < W && lane < cap) mbar_init(bars + CL_MAX_RING * w + lane, 1);
-  fence_barrier_init();
   __syncthreads();
   const ulonglong2* Kg = reinterpret_cast<const ulonglong2*>(S.kc) + (size_t)pa * CL_POS_F4;
   KPos kr[KREG ? KREG : 1];
@@ -957,8 +945,8 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
         kr[i].r[4 * q + 2] = v.z; kr[i].r[4 * q + 3] = v.w;
       }
     }
-  const int nkr = min(m, KREG), ntm = min(m - nkr, (tm_share - tm_m) / 36), ns = cap ? m - nkr - ntm : 0;
-  if (ns < m - nkr - ntm && lane == 0) atomicExch(flags + 1, 1);  // no launch of the plan's
+  const int nkr = min(m, KREG), ntm = min(m - nkr, (tm_share - tm_m) / 36);
+  const int ns = min(cap, m - nkr - ntm), ng = m - nkr - ntm - ns;
   Kg += (size_t)nkr * CL_POS_F4;
   const uint32_t tmw =
       tm_cols ? sh.tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)((w >> 2) * tm_share) : 0u;
@@ -975,20 +963,11 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
       for (int c = 0; c < 6; ++c) tm_st(tmm + M32_PACK * (t - ta) + 4 * c, __ldg(m2 + c));
     }
   tm_wait_st();
-  const bool ring = ns > cap;
-  unsigned long long* bar = bars + CL_MAX_RING * w;
   ulonglong2* Kw = Kres + (size_t)w * cap * CL_POS_F4;
-  auto fetch = [&](int pos, int sl) {  // one lane: the pos-th of the ns into slot sl
-    mbar_arrive_tx(bar + sl, CL_POS_BYTES);
-    bulk_g2s(Kw + (size_t)sl * CL_POS_F4, Kg + (size_t)(ntm + pos) * CL_POS_F4, CL_POS_BYTES,
-             bar + sl);
-  };
-  if (lane == 0)
-#pragma unroll 1
-    for (int k = 0; k < min(ns, cap); ++k) fetch(k, k);
-  int rslot = 0, rpos = ring ? cap : 0;  // the slot to read next, the position it then takes
-  unsigned rphase = 0u;                  // parity of the slots' phases, by slot
-  bool dry = false;                      // a copy did not arrive: no more waits or copies
+  Kg += (size_t)ntm * CL_POS_F4;
+#pragma unroll 4
+  for (int i = lane; i < ns * CL_POS_F4; i += 32) Kw[i] = __ldg(Kg + i);
+  Kg += (size_t)ns * CL_POS_F4;  // what streams
   // the vectors of a sweep under way
   {
     const float2* r2 = reinterpret_cast<const float2*>((const float*)S.r + 6 * (size_t)n0);
@@ -1031,7 +1010,6 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
   for (unsigned c = 0; !GRID && c < C; ++c)
     if (sh.wlo[c] < min(n, TILE * tb) && sh.whi[c] > TILE * ta && tb > ta) dest |= 1u << c;
 
-  int products = 0;  // matrix products of this launch
 #pragma unroll 1
   for (int step = 0; step < max_steps && state != ST_DONE && !(GRID && sh.lost); ++step) {
     float alpha = 0.f;
@@ -1085,40 +1063,6 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
         int t = ta, left = m ? toffS[ta - T0 + 1] - toffS[ta - T0] : 0;  // positions of the tile
         const uint16_t* sl = slot + 32 * (pa - U0) + lane;
         unsigned long long acc[3] = {0ull, 0ull, 0ull};
-        // starts the load of position i; a slot of the ring is refilled after it
-        auto load = [&](KPos& K, int i) {
-          if (i < ntm) {
-            tm_ld36(tmw + 36 * i, K.r);
-            return;
-          }
-          if (ring || products == 0) {  // (a resident slot is waited for once)
-            if (!dry && !mbar_wait(bar + rslot, (rphase >> rslot) & 1u)) {
-              dry = true;
-              atomicExch(flags + 1, 1);
-            }
-            dry = __any_sync(0xffffffffu, dry);
-          }
-          const uint4* kp = reinterpret_cast<const uint4*>(Kw + (size_t)rslot * CL_POS_F4) + lane;
-#pragma unroll
-          for (int q = 0; q < 9; ++q) {
-            const uint4 v = kp[32 * q];
-            K.r[4 * q] = v.x; K.r[4 * q + 1] = v.y; K.r[4 * q + 2] = v.z; K.r[4 * q + 3] = v.w;
-          }
-        };
-        // the slot of position i has been read
-        auto refill = [&](int i) {
-          if (i < ntm) return;
-          if (ring) {
-            rphase ^= 1u << rslot;
-            __syncwarp();
-            if (lane == 0 && !dry) {
-              fence_proxy_async();
-              fetch(rpos, rslot);
-            }
-            if (++rpos == ns) rpos = 0;
-          }
-          if (++rslot == min(cap, ns)) rslot = 0;
-        };
         auto row_end = [&] {
           if (--left) return;  // else the tile's rows are done
           const int l = TILE * t + lane - n0;
@@ -1150,17 +1094,50 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
         for (int i = 0; i < ntm + ns; ++i) {
           KPos K;
           float p[6];
-          load(K, i);
+          if (i < ntm) {
+            tm_ld36(tmw + 36 * i, K.r);
+          } else {
+            const uint4* kp = reinterpret_cast<const uint4*>(Kw + (size_t)(i - ntm) * CL_POS_F4) + lane;
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+              const uint4 v = kp[32 * q];
+              K.r[4 * q] = v.x; K.r[4 * q + 1] = v.y; K.r[4 * q + 2] = v.z; K.r[4 * q + 3] = v.w;
+            }
+          }
           const bool real = column(p);
           if (i < ntm) tm_wait_ld();
           tm_loaded(K.r);
           if (real) fma_pos(K, p, acc);
-          refill(i);
           row_end();
           __syncwarp();
         }
+        if (ng > 0) {
+          const ulonglong2* kp = Kg + lane;
+          ulonglong2 k[9];
+#pragma unroll
+          for (int q = 0; q < 9; ++q) k[q] = __ldg(kp + 32 * q);
+#pragma unroll 1
+          for (int i = 1; i <= ng; ++i) {
+            float p[6];
+            const bool real = column(p);
+            if (i < ng) kp += CL_POS_F4;  // (the last position is loaded again, and not used)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+              unsigned long long s = acc[a];
+#pragma unroll
+              for (int q = 0; q < 3; ++q) {
+                s = fma2(k[3 * a + q].x, pack2(p[2 * q], p[2 * q]), s);
+                s = fma2(k[3 * a + q].y, pack2(p[2 * q + 1], p[2 * q + 1]), s);
+              }
+              if (real) acc[a] = s;
+#pragma unroll
+              for (int q = 0; q < 3; ++q) k[3 * a + q] = __ldg(kp + 32 * (3 * a + q));
+            }
+            row_end();
+            __syncwarp();
+          }
+        }
       }
-      ++products;
       // p^T q: four lanes per 5-node group (six groups a tile): lane j forms the
       // levels 16, 8 and 4 of the tree over the rows l = j mod 4 of the group's
       // 30 (lanes 30 and 31 of that tree hold zero), two shuffles the last two
@@ -1578,11 +1555,6 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
       sts6((float*)S.z + 6 * (size_t)i, z);
     }
   }
-  // the ring's copies in flight land before the shared memory is released
-  if (lane == 0)
-#pragma unroll 1
-    for (int k = 0; k < min(ns, cap); ++k)
-      if (ring || products == 0) mbar_wait(bar + k, (rphase >> k) & 1u);
   if (tm_cols && w == 0) tm_free(sh.tmem, tm_cols);
   if (!GRID) cl_sync();  // no CTA leaves while another may still store into it
   if (rank == 0 && tid == 0 && !lost) {
@@ -1610,7 +1582,7 @@ size_t cluster_smem_bytes(const ClusterShare& c, int precond, bool m_tm, bool te
   s += (team ? 1 : 2) * a(24 * (size_t)c.window) + 3 * a(24 * own) + 8 * WARPS * nt + 32 * nt;
   if (!m_tm) s += (precond == SSO_JACOBI ? 768 : 3072) * nt;
   s += 64 * (size_t)c.positions + a(4 * (nt + 1));
-  return s + 8 * CL_MAX_RING * (CL_MAX_THREADS / 32) + 128;
+  return s + 128;
 }
 
 // Columns of tensor memory for a CTA of `smem` bytes of dynamic shared memory:
