@@ -237,6 +237,8 @@ struct sso_model {
   bool cluster_ok = false;
   int cl_positions = 0;
   ClusterShare cl_share[CL_SIZES] = {}, cl_team[CL_TEAMS] = {};
+  // FP64 teams of k + 1 tiles a CTA (n_tiles 0: too many CTAs)
+  ClusterShare cl_team64[TEAM64_TILES] = {};
   int* d_toff;
   bool is_chain = false;
   int* d_chain_up;        // [n_nodes] block (i, i+1) or -1
@@ -1246,6 +1248,78 @@ sso_status launch_bins(sso_batch* B, const std::vector<ClusterBin>& bins, const 
 // its completion; other kernels beside them end by themselves).
 std::mutex g_team_mutex;
 
+// FP64 CG on teams (Jacobi and block Jacobi): one launch of systems with teams
+// of one size.
+struct Team64Bin {
+  int first, n, team, threads, smem;
+};
+
+// Sorts the active systems into launches; *fits is false when one does not fit
+// (the batch then runs the two-kernel engine).  Tiles per CTA by the least
+// estimated time of all: an iteration is the barriers and sums (12,000 clocks),
+// plus the FP64 pipe's work on a tile (7,000) and K from L2 where it does not
+// fit shared memory; systems beyond those resident at once run in waves.
+// Measured (us an iteration of all, estimate in brackets at 1.92 GHz): one 41 x
+// 41 grid shell 11.6 (9.9), 16 of them 31.0 (28.1), 64 123 (121).  Teams were
+// faster than the two kernels at every size and count tried (10 x 10 to 100 x
+// 100, 1 to 64 systems), so that whatever fits takes them.
+template <class GetModel>
+sso_status plan_team64(int n_sys, const std::vector<char>& active, bool jacobi, GetModel model,
+                       std::vector<int>& list, std::vector<Team64Bin>& bins, bool* fits) {
+  *fits = false;
+  list.clear();
+  bins.clear();
+  const ClusterDevice* dev = nullptr;
+  sso_status st = cluster_device(&dev);
+  if (st != SSO_OK) return st;
+  int n_act = 0;
+  for (int s = 0; s < n_sys; ++s) n_act += active[s] != 0;
+  struct Choice {
+    int sys, team, threads, smem;
+  };
+  std::vector<Choice> choice;
+  for (int s = 0; s < n_sys; ++s) {
+    if (!active[s]) continue;
+    const sso_model* M = model(s);
+    Choice best{s, 0, 0, 0};
+    double best_t = HUGE_VAL;
+    for (int k = 0; k < TEAM64_TILES; ++k) {
+      const ClusterShare& sh = M->cl_team64[k];
+      const int C = (M->n_tiles + k) / (k + 1);
+      if (!sh.n_tiles || C > dev->ctas) continue;
+      size_t k_bytes = 0;
+      const size_t need = team64_smem_bytes(sh, jacobi, &k_bytes);
+      if (need > (size_t)dev->smem) continue;
+      const bool k_in = need + k_bytes <= (size_t)dev->smem;
+      const int per = std::min(dev->ctas / C, CL_MAX_TEAMS);
+      const double t = 12000.0 + 7000.0 * sh.own_tiles + (k_in ? 0.0 : k_bytes / 64.0);
+      const double all = t * ((n_act + per - 1) / per);
+      if (all < best_t) {
+        best_t = all;
+        best = {s, C, std::min(TEAM64_THREADS, 32 * WARPS * sh.own_tiles),
+                (int)(need + (k_in ? k_bytes : 0))};
+      }
+    }
+    if (!best.team) return SSO_OK;
+    choice.push_back(best);
+  }
+  std::stable_sort(choice.begin(), choice.end(),
+                   [](const Choice& a, const Choice& b) { return a.team > b.team; });
+  for (size_t i = 0; i < choice.size(); ++i) {
+    const Choice& c = choice[i];
+    const int per = std::min(dev->ctas / c.team, CL_MAX_TEAMS);
+    if (bins.empty() || bins.back().team != c.team || bins.back().n == per)
+      bins.push_back({(int)i, 0, c.team, 0, 0});
+    Team64Bin& b = bins.back();
+    ++b.n;
+    b.threads = std::max(b.threads, c.threads);
+    b.smem = std::max(b.smem, c.smem);
+    list.push_back(c.sys);
+  }
+  *fits = !list.empty();
+  return SSO_OK;
+}
+
 // CG steps of a system per launch: long enough that loading a system (some
 // microseconds) does not count, short enough that the host sees finished
 // systems and the wall-clock cap within a few milliseconds.
@@ -1271,9 +1345,15 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
   // runs time the two-kernel engine's launches
   bool cluster = false;
   std::vector<ClusterBin> bins;
+  std::vector<Team64Bin> bins64;
   if (o->precision == SSO_FP32_IR && !B->profiling) {
     sso_status st = plan_bins(B->n_sys, active, o->precond, 1, true,
                               [B](int s) { return B->models[s]; }, B->h_list, bins, &cluster);
+    if (st != SSO_OK) return st;
+  }
+  if (fp64 && !B->profiling && (o->precond == SSO_JACOBI || o->precond == SSO_BLOCK_JACOBI)) {
+    sso_status st = plan_team64(B->n_sys, active, o->precond == SSO_JACOBI,
+                                [B](int s) { return B->models[s]; }, B->h_list, bins64, &cluster);
     if (st != SSO_OK) return st;
   }
   int n_act = 0;
@@ -1335,17 +1415,23 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
                        cudaMemcpyHostToDevice, B->stream));
     int max_nodes = 1;
     for (int s : B->h_list) max_nodes = std::max(max_nodes, B->models[s]->n_nodes);
-    CL(launch_cluster_pack(B->d_sys, B->d_list, (int)B->h_list.size(), max_nodes, B->stream), 1);
+    if (!fp64)
+      CL(launch_cluster_pack(B->d_sys, B->d_list, (int)B->h_list.size(), max_nodes, B->stream),
+         1);
     const int steps = o->timeout_ms > 0.0 ? std::min(kClusterSteps, o->iters_per_launch)
                                           : kClusterSteps;
     const long long max_launches = (2LL * o->max_iter + 4LL * o->max_sweeps) / steps + 8;
-    const bool teams = std::any_of(bins.begin(), bins.end(),
-                                   [](const ClusterBin& b) { return b.team; });
+    const bool teams = fp64 || std::any_of(bins.begin(), bins.end(),
+                                           [](const ClusterBin& b) { return b.team; });
     for (long long launches = 1;; ++launches) {
       std::unique_lock<std::mutex> lock(g_team_mutex, std::defer_lock);
       if (teams) lock.lock();
       sso_status st = launch_bins(B, bins, B->d_list, o->precond, steps);
       if (st != SSO_OK) return st;
+      for (const Team64Bin& b : bins64)
+        CL(launch_team64(B->d_sys, B->d_list + b.first, b.n, b.team, b.threads, b.smem,
+                         o->precond == SSO_JACOBI, B->d_slots, B->d_n_active, steps, B->stream),
+           1);
       CK(cudaMemcpyAsync(B->h_flag + 2, B->d_n_active, 2 * sizeof(int), cudaMemcpyDeviceToHost,
                          B->stream));
       CK(cudaEventRecord(B->ev, B->stream));
@@ -1567,7 +1653,6 @@ void plan_cluster(sso_model* M, const HostTopo& T) {
   M->cl_positions = T.toff[M->n_tiles];
   const size_t room = (size_t)std::max(M->n_eb, M->n_blocks) * 36 * sizeof(double);
   M->cluster_ok = n_chunks_of(M) <= CL_MAX_CHUNKS && cluster_pack_bytes(M) <= room;
-  if (!M->cluster_ok) return;
   auto share = [&](int C) {
     int win = 0, pos = 0;
     for (int r = 0; r < C; ++r) {  // the kernel's split of the tiles
@@ -1590,6 +1675,19 @@ void plan_cluster(sso_model* M, const HostTopo& T) {
     }
     return ClusterShare{M->n_tiles, (M->n_tiles + C - 1) / C, win, pos, members};
   };
+  for (int k = 0; k < TEAM64_TILES && n_chunks_of(M) <= CL_MAX_CHUNKS; ++k) {
+    const int C = (M->n_tiles + k) / (k + 1);
+    if (C > cl_team_of(0)) continue;
+    M->cl_team64[k] = share(C);
+    int blocks = 0;
+    for (int r = 0; r < C; ++r) {
+      const int t0 = (int)((long long)M->n_tiles * r / C);
+      const int t1 = (int)((long long)M->n_tiles * (r + 1) / C);
+      blocks = std::max(blocks, T.row_ptr[std::min(n, TILE * t1)] - T.row_ptr[std::min(n, TILE * t0)]);
+    }
+    M->cl_team64[k].members = blocks;
+  }
+  if (!M->cluster_ok) return;
   for (int k = 0; k < CL_SIZES; ++k) M->cl_share[k] = share(cl_size_of(k));
   for (int k = 0; k < CL_TEAMS; ++k) M->cl_team[k] = share(cl_team_of(k));
 }

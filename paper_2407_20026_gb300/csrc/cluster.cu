@@ -10,8 +10,8 @@
 // all, three times HBM, while the systems in flight fit its 126 MB), and the
 // CTAs meet at two cluster barriers an iteration (about 0.25 us each).
 // Measured, 64 x 64 shells (25,350 DOF) to 1e-6, two-kernel engine -> here:
-// one system 16.1 -> 7.0 us an iteration (208.8 -> 90.2 ms a solve; on 16 SMs),
-// 48 systems 1.58 -> 0.71 us a system-iteration (945 -> 424 ms); two-level
+// one system 16.1 -> 6.5 us an iteration (208.8 -> 83.6 ms a solve; on 16 SMs),
+// 48 systems 1.58 -> 0.66 us a system-iteration (945 -> 393 ms); two-level
 // preconditioner, one 28.8 -> 14.2 us, 128 systems 403 -> 256 ms.
 //
 // Larger systems (and a few middle-sized ones together) take teams of 152, 76
@@ -19,8 +19,8 @@
 // stream the rest, but z goes through global memory and the barriers too
 // (team_sync: 4,000 to 6,000 clocks an iteration more than a cluster's).
 // Measured, us an iteration, two-kernel engine -> team: 256 x 256 shell
-// (396,294 DOF, K 85 MB, 57 MB of it streamed) 36 -> 13.6, 128 x 128 shell
-// 28 -> 8.7, 100 x 100 grid shell 25 -> 8.0 (on a cluster of 16: 13.8).  The
+// (396,294 DOF, K 85 MB, 57 MB of it streamed) 36 -> 12.5, 128 x 128 shell
+// 28 -> 8.2, 100 x 100 grid shell 25 -> 7.6 (on a cluster of 16: 13.8).  The
 // coarse correction needs a cluster: two-level systems do not take teams.
 //
 // The arithmetic is the two-kernel engine's, so every result is the same bits
@@ -368,7 +368,7 @@ __device__ __noinline__ Fix fix_total(const Fix* slot, int n, int lane) {
 // clocks (3,000 with data's fences), this 1,800 to 2,200; a slot per CTA that
 // all poll 6,200, a mailbox per CTA that all store into 4,700, clusters of 4
 // and their mailboxes 3,700.  256 x 256 shell, us an iteration: slots 21,
-// mailboxes 15.9, this 13.6.
+// mailboxes 15.9, this 13.6 (12.5 since K streams through registers).
 // A CTA that waits for some seconds gives up: it sets the error flag, and its
 // later barriers do not wait.
 constexpr int kTeamPolls = 1 << 23;  // of about 700 clocks: some seconds
@@ -927,7 +927,9 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
   // shared memory, and the others come from L2 in every iteration, by plain
   // loads that run three thirds of a position ahead of the products (the
   // registers of a third are loaded again as soon as it has been used).  (A
-  // ring of slots in shared memory that bulk copies refill: XXX)
+  // ring of slots in shared memory that bulk copies refill waited for each copy
+  // in turn: 48 systems 421 ms against 393, 256 x 256 shell 13.8 us an iteration
+  // against 12.5; slots of a third of a position: 509 ms, 15.1 us.)
   const int ta = w < W ? T0 + nt * w / W : T1, tb = w < W ? T0 + nt * (w + 1) / W : T1;
   const int pa = __ldg(S.toff + ta), m = __ldg(S.toff + tb) - pa;
   if (tm_cols && w == 0) tm_alloc(&sh.tmem, tm_cols);
@@ -1569,6 +1571,250 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
   }
 }
 
+// The FP64 CG of a system on one team of CTAs (cooperative launch), up to
+// max_steps steps from the state in its SysScalars, as cluster_cg_kernel for
+// the FP32 one and with the arithmetic and trees of the two-kernel engine
+// (pcg_a_kernel<double>, pcg_b_kernel<double>): the same bits.
+//
+// What bounds it: the FP64 pipe, two multiply-adds a clock and SM, and the
+// latency of two barriers and the FP64 sums after each.  The two-kernel engine
+// forms p = z + beta p again for every block of every row, which doubles the
+// pipe's work; here a CTA updates its window of p once, in shared memory, with
+// its rows of the other vectors, M and (where it fits) K.  A CTA has few tiles,
+// six warps on each: a lane per row (five nodes a warp) for the products and
+// the updates, a lane per node for the dot products' trees.
+// Measured, us an iteration, two kernels -> here: 41 x 41 grid shell (10,086 DOF)
+// 26.8 -> 11.6, 100 x 100 39 -> 22.8, 24 x 24 shell 26 -> 12.5; with two kernels
+// under per-launch timing: 64 grid shells of 41 x 41 172 -> 123.
+template <bool JAC>
+__global__ void __launch_bounds__(TEAM64_THREADS, 1) team64_kernel(
+    const SysDesc* __restrict__ sys, const int* __restrict__ list, int* __restrict__ flags,
+    int max_steps, int smem_bytes, int team, unsigned long long* slots) {
+  extern __shared__ __align__(16) unsigned char cl_smem[];
+  __shared__ ClShared sh;
+  const int C = team, rank = (int)blockIdx.x % C;
+  const int tid = threadIdx.x, nth = blockDim.x, w = tid >> 5, lane = tid & 31, W = nth >> 5;
+  {
+    const SysDesc& G = sys[list[blockIdx.x / C]];
+    if (*(volatile const int*)&G.sc->state == ST_DONE) return;  // alike in every CTA
+    for (int i = tid; i < (int)(sizeof(SysDesc) / 4); i += nth)
+      reinterpret_cast<int*>(&sh.sys)[i] = reinterpret_cast<const int*>(&G)[i];
+    for (int i = tid; i < (int)(sizeof(SysScalars) / 4); i += nth)
+      reinterpret_cast<int*>(&sh.sc)[i] = __ldcg(reinterpret_cast<const int*>(G.sc) + i);
+  }
+  if (tid == 0) {
+    sh.n_done = 1;
+    sh.lo = INT_MAX;
+    sh.hi = 0;
+    sh.epoch = 0u;
+    sh.lost = 0;
+    sh.team = team;
+    sh.copy = rank % CL_TEAM_COPIES;
+    sh.slots = slots + CL_TEAM_WORDS * (blockIdx.x / C);
+    sh.flags = flags;
+  }
+  if (tid < 12) sh.before[tid / 6][tid % 6] = 0ull;
+  for (int i = tid; i < 96; i += nth) sh.words[i / 6][i % 6] = 0ull;
+  __syncthreads();
+  const SysDesc& S = sh.sys;
+  const int n = S.n_nodes, n_tiles = S.n_tiles, n_ow = WARPS * n_tiles, n_vw = (n_ow + 255) / 256;
+  const int T0 = n_tiles * rank / C, T1 = n_tiles * (rank + 1) / C, nt = T1 - T0;
+  const int n0 = min(n, TILE * T0), n1 = min(n, TILE * T1), nown = n1 - n0;
+  const int j0 = __ldg(S.row_ptr + n0), nb = __ldg(S.row_ptr + n1) - j0;
+  {
+    int lo = INT_MAX, hi = 0;
+    for (int i = n0 + tid; i < n1; i += nth) {
+      lo = min(lo, __ldg(S.col + __ldg(S.row_ptr + i)));
+      hi = max(hi, __ldg(S.col + __ldg(S.row_ptr + i + 1) - 1) + 1);
+    }
+    if (hi > lo) {
+      atomicMin(&sh.lo, lo);
+      atomicMax(&sh.hi, hi);
+    }
+  }
+  __syncthreads();
+  const int lo = nown ? sh.lo : 0, wn = nown ? sh.hi - sh.lo : 0;
+  // shared memory (team64_smem_bytes is the same sum)
+  double* P = reinterpret_cast<double*>(cl_smem);      // the window's p
+  double* Q = P + 6 * (size_t)wn;                      // own rows
+  double* R = Q + 6 * (size_t)nown;
+  double* X = R + 6 * (size_t)nown;
+  double* Z = X + 6 * (size_t)nown;
+  double* Ms = Z + 6 * (size_t)nown;
+  double* Ks = Ms + (JAC ? 6 : 36) * (size_t)nown;
+  const size_t used = (size_t)((unsigned char*)Ks - cl_smem) + 4 * ((size_t)nb + nown + 2);
+  const bool k_in = used + 288 * (size_t)nb <= (size_t)smem_bytes;
+  int* slot = reinterpret_cast<int*>(Ks + (k_in ? 36 * (size_t)nb : 0));  // 6 x window slot
+  int* rp = slot + nb;
+  const double* Mg = S.M64 + (JAC ? 6 : 36) * (size_t)n0;
+  for (int i = tid; i < (JAC ? 6 : 36) * nown; i += nth) Ms[i] = __ldg(Mg + i);
+  const double* Kg = S.K64 + 36 * (size_t)j0;
+  if (k_in)
+    for (int i = tid; i < 18 * nb; i += nth)
+      reinterpret_cast<double2*>(Ks)[i] = __ldg(reinterpret_cast<const double2*>(Kg) + i);
+  const double* K = k_in ? Ks : Kg;
+  for (int i = tid; i < nb; i += nth) slot[i] = 6 * (__ldg(S.col + j0 + i) - lo);
+  for (int i = tid; i <= nown; i += nth) rp[i] = __ldg(S.row_ptr + n0 + i) - j0;
+  for (int i = tid; i < 6 * nown; i += nth) {
+    R[i] = __ldcg((const double*)S.r + 6 * (size_t)n0 + i);
+    X[i] = __ldcg(S.x + 6 * (size_t)n0 + i);
+  }
+  {
+    const double* pg = (const double*)(sh.sc.parity ? S.p1 : S.p0) + 6 * (size_t)lo;
+    for (int i = tid; i < 6 * wn; i += nth) P[i] = __ldcg(pg + i);
+  }
+  bool z_alt = false;  // z is in S.zb, not S.z
+  // this lane's row within a group of five nodes
+  const int ln = lane / 6, rr = lane % 6;
+  __syncthreads();
+
+  int state = sh.sc.state;
+  for (int step = 0; step < max_steps && state != ST_DONE && !sh.lost; ++step) {
+    if (state == ST_PCG) {
+      const bool first = sh.sc.inner == 0;
+      const double beta = first ? 0.0 : sh.sc.beta;
+      const double* z = (const double*)(z_alt ? S.zb : S.z) + 6 * (size_t)lo;
+      for (int i = tid; i < 6 * wn; i += 4 * nth) {
+        double v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (i + u * nth < 6 * wn) v[u] = __ldcg(z + i + u * nth);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (i + u * nth < 6 * wn)
+            P[i + u * nth] = fma(beta, first ? v[u] : P[i + u * nth], v[u]);
+      }
+      __syncthreads();
+      for (int g = w; g < WARPS * nt; g += W) {
+        const int l = NODES_PER_WARP * g + ln;
+        double part = 0.0;
+        if (lane < 6 * NODES_PER_WARP && l < nown) {
+          double acc = 0.0;
+          const int e = rp[l + 1];
+          for (int j = rp[l]; j < e; ++j) {
+            const double2* kv = reinterpret_cast<const double2*>(K + 36 * (size_t)j + 6 * rr);
+            const double2* pv = reinterpret_cast<const double2*>(P + slot[j]);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+              const double2 a = kv[q], b = pv[q];
+              acc = fma(a.x, b.x, acc);
+              acc = fma(a.y, b.y, acc);
+            }
+          }
+          Q[6 * l + rr] = acc;
+          part = P[6 * (n0 - lo + l) + rr] * acc;
+        }
+        part = warp_sum(part);
+        if (lane == 0) S.part_a[WARPS * T0 + g] = part;
+      }
+      team_sync(sh, true);
+      for (int v = w; v < n_vw; v += W) {
+        const double a = vwarp_sum(S.part_a, v, n_ow, lane);
+        if (lane == 0) sh.red[v] = a;
+      }
+      __syncthreads();
+      if (tid == 0)
+        finish_a_scalars(&sh.sc, ST_PCG, total_a(sh.red, n_vw, S.n_chunks), 0.0, &sh.n_done);
+      __syncthreads();
+      if (sh.sc.state == ST_DONE) {
+        state = ST_DONE;
+        break;
+      }
+    } else {  // INIT, RESID
+      residual_phase(S, state, WARPS * T0, WARPS * T1, n1, n_ow);
+      team_sync(sh, true);
+      for (int v = w; v < 2 * n_vw; v += W) {
+        const bool second = v >= n_vw;
+        const int k = second ? v - n_vw : v;
+        const double a = vwarp_sum(S.part_a + (second ? n_ow : 0), k, n_ow, lane);
+        if (lane == 0) sh.red[(second ? CL_MAX_VWARPS : 0) + k] = a;
+      }
+      __syncthreads();
+      if (tid == 0) residual_scalars(sh, state, n_vw, S.n_chunks);
+      __syncthreads();
+      const double rr64 = sh.sc.rr64;
+      if (!(f64_finite(rr64) && !(rr64 <= sh.sc.rtol2 * sh.sc.ff))) {
+        __syncthreads();
+        if (tid == 0) finish_b(&sh.sc, state, 0.0, 0.0, &sh.n_done, false);
+        __syncthreads();
+        state = sh.sc.state;
+        continue;
+      }
+    }
+    const double alpha = sh.sc.alpha, ua = alpha * sh.sc.scale;
+    const double inv_norm = state == ST_PCG ? 0.0 : 1.0 / ::sqrt(sh.sc.rr64);
+    double* zn = (double*)(z_alt ? S.z : S.zb) + 6 * (size_t)n0;
+    for (int g = w; g < WARPS * nt; g += W) {
+      const int l = NODES_PER_WARP * g + ln, i = 6 * l + rr;
+      const bool act = lane < 6 * NODES_PER_WARP && l < nown;
+      if (act) {
+        if (state == ST_PCG) {
+          X[i] = fma(ua, P[6 * (n0 - lo) + i], X[i]);
+          R[i] = fma(-alpha, Q[i], R[i]);
+        } else {
+          R[i] = __ldcg(S.r64 + 6 * (size_t)n0 + i) * inv_norm;
+        }
+      }
+      __syncwarp();
+      if (act) {
+        double z;
+        if (JAC) {
+          z = Ms[i] * R[i];
+        } else {
+          z = 0.0;
+#pragma unroll
+          for (int c = 0; c < 6; ++c) z = fma(Ms[36 * l + 6 * rr + c], R[6 * l + c], z);
+        }
+        Z[i] = z;
+        zn[i] = z;
+      }
+    }
+    __syncthreads();
+    // r^T z and r^T r of a tile: a warp each
+    for (int k = w; k < 2 * nt; k += W) {
+      const int l = TILE * (k >> 1) + lane;
+      double v = 0.0;
+      if (lane < TILE && l < nown) {
+        const double* b = k & 1 ? R : Z;
+#pragma unroll
+        for (int a = 0; a < 6; ++a) v = fma(R[6 * l + a], b[6 * l + a], v);
+      }
+      v = warp_sum(v);
+      if (lane == 0) S.part_b[(k & 1) * n_tiles + T0 + (k >> 1)] = v;
+    }
+    z_alt = !z_alt;
+    team_sync(sh, true);
+    if (w < 2) {
+      const double v = total_b(S.part_b + (size_t)w * n_tiles, n_tiles, S.n_chunks, lane,
+                               sh.red + CL_MAX_VWARPS + CL_MAX_CHUNKS * w);
+      if (lane == 0) (w == 0 ? sh.ex_rz : sh.ex_rr) = v;
+    }
+    __syncthreads();
+    if (tid == 0) finish_b(&sh.sc, state, sh.ex_rz, sh.ex_rr, &sh.n_done, false);
+    __syncthreads();
+    state = sh.sc.state;
+    if (state == ST_RESID) {  // the other CTAs read x next
+      for (int i = tid; i < 6 * nown; i += nth) S.x[6 * (size_t)n0 + i] = X[i];
+      team_sync(sh, true);
+    }
+  }
+  if (sh.lost) return;  // a barrier gave up: the run has failed
+  if (state == ST_PCG || state == ST_DONE)
+    for (int i = tid; i < 6 * nown; i += nth) S.x[6 * (size_t)n0 + i] = X[i];
+  if (state == ST_PCG) {
+    double* pg = (double*)(sh.sc.parity ? S.p1 : S.p0) + 6 * (size_t)n0;
+    for (int i = tid; i < 6 * nown; i += nth) {
+      ((double*)S.r)[6 * (size_t)n0 + i] = R[i];
+      ((double*)S.z)[6 * (size_t)n0 + i] = Z[i];
+      pg[i] = P[6 * (n0 - lo) + i];
+    }
+  }
+  if (rank == 0 && tid == 0) {
+    *S.sc = sh.sc;
+    if (state == ST_DONE) atomicSub(flags, 1);
+  }
+}
+
 }  // namespace
 
 // Shared memory of one CTA before resident K (the kernel carves the same sum).
@@ -1605,7 +1851,8 @@ static cudaError_t cluster_attributes(int* max_smem) {
   static int limit = 0;
   std::lock_guard<std::mutex> lock(mu);
   if (!limit) {
-    const void* fns[9] = {(const void*)cluster_cg_kernel<false, false, 0, false>,
+    const void* fns[11] = {(const void*)team64_kernel<false>, (const void*)team64_kernel<true>,
+                          (const void*)cluster_cg_kernel<false, false, 0, false>,
                           (const void*)cluster_cg_kernel<false, true, 0, false>,
                           (const void*)cluster_cg_kernel<true, false, 0, false>,
                           (const void*)cluster_cg_kernel<false, false, CL_KREG, false>,
@@ -1717,6 +1964,35 @@ cudaError_t launch_cluster_cg(const SysDesc* sys, const int* list, int n_list, i
                                  : run(cluster_cg_kernel<false, false, CL_KREG, false>);
   return precond == SSO_JACOBI ? run(cluster_cg_kernel<false, true, 0, false>)
                                : run(cluster_cg_kernel<false, false, 0, false>);
+}
+
+// The shared memory of a CTA of the FP64 engine without K, and all of K's.
+size_t team64_smem_bytes(const ClusterShare& c, bool jacobi, size_t* k_bytes) {
+  const size_t own = (size_t)TILE * c.own_tiles;
+  *k_bytes = 288 * (size_t)c.members;
+  return 48 * (size_t)c.window + 48 * 4 * own + 8 * (jacobi ? 6 : 36) * own +
+         4 * ((size_t)c.members + own + 2);
+}
+
+cudaError_t launch_team64(const SysDesc* sys, const int* list, int n_list, int team, int threads,
+                          int smem, bool jacobi, unsigned long long* slots, int* flags,
+                          int max_steps, cudaStream_t s) {
+  if (n_list <= 0) return cudaSuccess;
+  int limit = 0;
+  cudaError_t e = cluster_attributes(&limit);
+  if (e != cudaSuccess) return e;
+  if (smem > limit || n_list > CL_MAX_TEAMS || threads > TEAM64_THREADS)
+    return cudaErrorInvalidValue;
+  e = cudaMemsetAsync(slots, 0, CL_SLOT_BYTES, s);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at[1];
+  cluster_config(cfg, at, n_list, team, threads, smem, s);
+  at[0] = cudaLaunchAttribute{};
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  return cudaLaunchKernelEx(&cfg, jacobi ? team64_kernel<true> : team64_kernel<false>, sys, list,
+                            flags, max_steps, smem, team, slots);
 }
 
 }  // namespace sso

@@ -179,3 +179,27 @@ def test_teams_many_launches_and_adjoint(sso):
     assert np.array_equal(cut[1][0]["u"], whole[1][0]["u"])
     g = np.random.default_rng(3).standard_normal(6 * m["xyz"].shape[0])
     _same(sso, [m], g=[g], rtol=1e-6, max_iter=600)
+
+
+@pytest.mark.parametrize("precond", ["jacobi", "block_jacobi"])
+@pytest.mark.parametrize("n", [2, 29, 30, 31, 61, 4591])
+def test_fp64_tile_edges(sso, n, precond):
+    # 4,591 nodes: 154 tiles, more than one on some CTAs
+    _same(sso, [_strip(n)], precision="fp64", precond=precond, rtol=1e-10, max_iter=400)
+
+
+@pytest.mark.parametrize("precond", ["jacobi", "block_jacobi"])
+def test_fp64_batches_launches_and_adjoint(sso, precond):
+    kw = dict(precision="fp64", precond=precond, rtol=1e-10, max_iter=500)
+    one = meshgen.shell(24, seed=2)  # K beyond a CTA's shared memory where CTAs are few
+    g = np.random.default_rng(3).standard_normal(6 * one["xyz"].shape[0])
+    _same(sso, [one], g=[g], **kw)
+    _same(sso, [meshgen.gridshell(41, seed=1)] * 3 + [meshgen.shell(9), meshgen.gridshell(75)], **kw)
+    _same(sso, [meshgen.shell(16, seed=s) for s in range(24)], **kw)
+    whole = _run(sso, [one], False, **kw)
+    cut = _run(sso, [one], False, timeout_ms=6e4, iters_per_launch=7, **kw)
+    assert cut[0][0]["iterations"] == whole[0][0]["iterations"]
+    assert np.array_equal(cut[1][0]["u"], whole[1][0]["u"])
+    warm = sso.Model(meshgen.gridshell(20))
+    warm.solve(precision="fp64", precond=precond, rtol=1e-6)
+    assert warm.solve(precision="fp64", precond=precond, rtol=1e-10, warm_start=1)["status"] == 0
