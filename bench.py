@@ -14,7 +14,9 @@ resident in HBM; `e2e` is the same through the C-ABI from host buffers
 (design upload and result download inside the timed region).  `roofline`
 reports the dominant kernel (CG kernel A: the FP32 BSR SpMV, or the FP64
 residual SpMV in refinement passes), timed live with CUDA events on the
-library's stream.  `--impl reference` times the FP64 CPU oracle on the same
+library's stream in one more, untimed step: a profiled step runs the engine
+of two kernels an iteration, which large systems take; the timed steps run one
+thread-block cluster per design with K on chip and in L2.  `--impl reference` times the FP64 CPU oracle on the same
 workload instead.
 """
 import argparse
@@ -1148,16 +1150,19 @@ def main():
                 "alg_bytes_per_cg_launch": B * bytes_pcg,
                 "launches_timed": a_launches, "kernel_ms_total": ms_a,
                 "kernel_b_ms_total": ms_b,
-                "kernel_times_from": "profiled step: events around every CG launch, the "
-                                     "batch run whole (the timed steps run it as two "
-                                     "concurrent halves)" if B >= 32 else "profiled step",
+                "kernel_times_from": "profiled step: events around every launch of the engine "
+                                     "of two kernels an iteration, the batch run whole (the "
+                                     "timed steps run clusters, which stream no K from HBM)",
                 # the timed steps as a whole: the algorithmic bytes of both CG
                 # kernels over the steps' elapsed time (everything else counted
-                # as time), against the same peak
+                # as time), against the same peak; above 1 where K is read from
+                # the chip and L2 instead
                 "step_hbm": {
                     "achieved": step_gbs, "frac": step_gbs / peak_gbs,
                     "bytes": step_bytes, "note": "kernel A (SpMV, FP64 residual passes) and "
-                                                 "kernel B (264 B per node) per CG iteration"},
+                                                 "kernel B (264 B per node) per CG iteration; not "
+                                                 "HBM traffic: the timed steps read K on "
+                                                 "chip and from L2"},
             },
             # elapsed per phase of the profiled step; each set-up stage is
             # one launch for the whole batch

@@ -123,7 +123,9 @@ typedef struct {
                                 such a sweep ends the solve with SSO_ERR_NOT_CONVERGED) */
   int32_t max_iter;          /* cap on CG iterations summed over sweeps */
   int32_t max_sweeps;        /* cap on refinement sweeps (FP64 residual recomputations) */
-  int32_t iters_per_launch;  /* CG iterations per captured CUDA-graph launch */
+  int32_t iters_per_launch;  /* CG iterations per captured CUDA-graph launch; engines that keep
+                                a system on chip make up to 1024 a launch (with timeout_ms:
+                                no more than iters_per_launch; in a server: four times it) */
   int32_t warm_start;        /* 1: start from the model's current u instead of 0 */
   double timeout_ms;         /* wall-clock cap, <= 0 for none */
 } sso_options;
@@ -281,15 +283,18 @@ sso_status sso_model_get_load(sso_model* model, double* f);
 
 /* ---------------------------------------------------------------------------
  * Batches: several models (any mix of sizes and topologies, all on the same
- * device) solved together.  Every CG iteration is one pass of two kernels over
- * all systems that are still iterating; each system keeps its own scalars,
+ * device) solved together.  Each system runs on a thread-block cluster, or on a
+ * team of CTAs of a cooperative launch (large systems, FP64); where a system of
+ * the batch fits neither, every CG iteration is one pass of two kernels over
+ * all systems that are still iterating.  Each system keeps its own scalars,
  * refinement state and convergence test, and its reductions follow a fixed
- * tiling of its own rows, so its result does not depend on which other systems
- * share the batch.  The batch runs on the stream of models[0].  A batch of 32
+ * tiling of its own rows, so its result depends neither on which other systems
+ * share the batch nor on which of these runs it.  Solves with teams of several
+ * batches of a process take turns.  The batch runs on the stream of models[0].  A batch of 32
  * or more models runs its CG as 2 to 4 parts at once (about 18,000 tiles of 30
  * nodes per part), on the streams of their first models and on as many host
- * threads (the first part on the calling thread); each part's kernel ramps and
- * tails overlap the others' work.  The results are the same bits as without
+ * threads (the first part on the calling thread); each part's launches overlap
+ * the others' tails.  The results are the same bits as without
  * the split (sso_batch_set_parts changes the count).
  */
 sso_status sso_batch_create(sso_model* const* models, int32_t n_models, sso_batch** out);
@@ -308,7 +313,8 @@ sso_status sso_batch_solve(sso_batch* batch, const sso_options* opts, sso_stats*
 sso_status sso_batch_gradient(sso_batch* batch, const double* w, const double* const* g,
                               sso_stats* stats);
 
-/* Kernel timing of the CG engine, for roofline measurements: while enabled,
+/* Kernel timing of the CG engine of two kernels an iteration, for roofline
+ * measurements: while enabled, every solve of this batch takes that engine, and
  * every CG kernel launch of this batch (kernel A: SpMV + p^T K p or the FP64
  * residual; kernel B: update + preconditioner) is bracketed by CUDA events on
  * the batch's stream and the durations are summed.  Enabling resets the sums.
@@ -338,8 +344,9 @@ sso_status sso_batch_setup_times(const sso_batch* batch, double* ms_elements,
  * are wanted.  A server keeps up to max_systems requests resident on the GPU
  * (their patterns, K, preconditioners and solver state), within
  * hbm_budget_bytes of per-request device memory and max_tiles tiles of 30
- * nodes.  Every sso_server_step runs one captured CUDA graph of CG iterations
- * over the resident systems; meanwhile it admits waiting requests as slots,
+ * nodes.  Every sso_server_step runs one launch of CG iterations (a cluster per
+ * resident system, or a captured CUDA graph of two kernels an iteration while
+ * one does not fit); meanwhile it admits waiting requests as slots,
  * tiles and budget allow (their element matrices, assembly and preconditioner
  * run on a second stream and overlap the CG), and when a system has converged
  * it computes its gradient, stores the result on the host and releases its

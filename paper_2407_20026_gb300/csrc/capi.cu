@@ -1059,14 +1059,17 @@ struct ClusterBin {
   bool team;  // teams of a cooperative launch, not clusters
 };
 
-// What the device holds at once (cluster_limits).
+// What the current device holds at once (cluster_limits).
 struct ClusterDevice {
   int smem = 0, slots[CL_SIZES], ctas = 0;
 };
 sso_status cluster_device(const ClusterDevice** out) {
   static std::mutex mu;
-  static ClusterDevice d;
+  static std::map<int, ClusterDevice> devices;
+  int dev = 0;
+  CK(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lock(mu);
+  ClusterDevice& d = devices[dev];
   if (!d.smem) {
     ClusterDevice q;
     CK(cluster_limits(&q.smem, q.slots, &q.ctas));

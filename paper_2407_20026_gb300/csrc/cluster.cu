@@ -54,6 +54,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <map>
 #include <mutex>
 
 #include "sso_internal.cuh"
@@ -1846,10 +1847,16 @@ int cluster_tm_positions(int smem, int own_tiles, int warps, bool m_tm) {
   return share < m ? -1 : (share - m) / 36;
 }
 
+// Sets the kernels' attributes on the current device, once (they are the
+// device's own); the dynamic shared memory of a CTA there.
 static cudaError_t cluster_attributes(int* max_smem) {
   static std::mutex mu;
-  static int limit = 0;
+  static std::map<int, int> limits;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
   std::lock_guard<std::mutex> lock(mu);
+  int& limit = limits[dev];
   if (!limit) {
     const void* fns[11] = {(const void*)team64_kernel<false>, (const void*)team64_kernel<true>,
                           (const void*)cluster_cg_kernel<false, false, 0, false>,
@@ -1861,10 +1868,8 @@ static cudaError_t cluster_attributes(int* max_smem) {
                           (const void*)cluster_cg_kernel<false, true, 0, true>,
                           (const void*)cluster_cg_kernel<false, false, CL_KREG, true>,
                           (const void*)cluster_cg_kernel<false, true, CL_KREG, true>};
-    int dev = 0, optin = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess)
-      e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    int optin = 0;
+    e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
     int room = optin;
     for (const void* f : fns) {
