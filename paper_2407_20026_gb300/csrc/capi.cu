@@ -1393,10 +1393,15 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
   CK(cudaMemcpyAsync(B->d_sc, B->h_sc, sizeof(SysScalars) * B->n_sys, cudaMemcpyHostToDevice,
                      B->stream));
   B->n_listed = B->n_sys;
-  B->h_flag[0] = n_act;
-  B->h_flag[1] = 0;
-  CK(cudaMemcpyAsync(B->d_n_active, B->h_flag, 2 * sizeof(int), cudaMemcpyHostToDevice,
-                     B->stream));
+  // (the one-CTA CG reads no flags, and its list is the identity that the
+  // batch keeps where every system is active: two copies fewer, about 3 us of
+  // a 1 ms evaluation of a 10 x 10 grid shell)
+  if (o->precision != SSO_F32X2) {
+    B->h_flag[0] = n_act;
+    B->h_flag[1] = 0;
+    CK(cudaMemcpyAsync(B->d_n_active, B->h_flag, 2 * sizeof(int), cudaMemcpyHostToDevice,
+                       B->stream));
+  }
   if (n_act > 0 && o->precision == SSO_F32X2) {
     // every active system's whole CG in one CTA of one launch
     B->h_list.clear();
@@ -1407,10 +1412,12 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
         groups = std::max(groups, (B->models[s]->n_nodes + NODES_PER_WARP - 1) / NODES_PER_WARP);
         max_nodes = std::max(max_nodes, B->models[s]->n_nodes);
       }
-    CK(cudaMemcpyAsync(B->d_list, B->h_list.data(), B->h_list.size() * sizeof(int),
-                       cudaMemcpyHostToDevice, B->stream));
+    const bool all = n_act == B->n_sys;
+    if (!all)
+      CK(cudaMemcpyAsync(B->d_list, B->h_list.data(), B->h_list.size() * sizeof(int),
+                         cudaMemcpyHostToDevice, B->stream));
     const int threads = 32 * std::min(32, groups);
-    CL(launch_small_cg(B->d_sys, B->d_list, (int)B->h_list.size(), threads, max_nodes,
+    CL(launch_small_cg(B->d_sys, all ? B->d_csys : B->d_list, (int)B->h_list.size(), threads, max_nodes,
                        o->precond == SSO_TWO_LEVEL, B->stream),
        2);
   } else if (n_act > 0 && cluster) {
@@ -2324,7 +2331,6 @@ sso_status create_batch(sso_model* const* models, int32_t n, sso_batch** out, bo
     D.zb = M->d_zb;
     D.klo = reinterpret_cast<float*>(M->d_ke);
     D.toff = M->d_toff;
-    D.kc = reinterpret_cast<float*>(M->d_ke);
     for (int k = 0; k < M->n_tiles; ++k) tiles.push_back(make_tile(M, s, k));
   }
   B->n_tiles = (int)tiles.size();
@@ -3138,7 +3144,6 @@ void fill_sysdesc(SysDesc& D, sso_model* M, int precond) {
   D.zb = M->d_zb;
   D.klo = reinterpret_cast<float*>(M->d_ke);
   D.toff = M->d_toff;
-  D.kc = reinterpret_cast<float*>(M->d_ke);
 }
 
 void init_scalars(SysScalars& S, const sso_options& o) {

@@ -10,8 +10,8 @@
 // all, three times HBM, while the systems in flight fit its 126 MB), and the
 // CTAs meet at two cluster barriers an iteration (about 0.25 us each).
 // Measured, 64 x 64 shells (25,350 DOF) to 1e-6, two-kernel engine -> here:
-// one system 16.1 -> 6.5 us an iteration (208.8 -> 83.6 ms a solve; on 16 SMs),
-// 48 systems 1.58 -> 0.66 us a system-iteration (945 -> 393 ms); two-level
+// one system 16.1 -> 6.5 us an iteration (208.8 -> 82.8 ms a solve; on 16 SMs),
+// 48 systems 1.58 -> 0.61 us a system-iteration (945 -> 377 ms); two-level
 // preconditioner, one 28.8 -> 14.2 us, 128 systems 403 -> 256 ms.
 //
 // Larger systems (and a few middle-sized ones together) take teams of 152, 76
@@ -47,7 +47,7 @@
 //
 // Two things cost more here than elsewhere: a spilled register (each barrier's
 // acquire drops L1, so that local memory is an L2 round trip: variants with
-// 300 bytes of spills ran at half the speed), and code (a warp walks through
+// 300 bytes of spills ran at half the speed, and the last 12 bytes cost 4 %), and code (a warp walks through
 // the whole iteration once, so that instructions come from the outer levels of
 // the instruction caches: loops are kept rolled, rare paths are functions).
 #include <math.h>
@@ -249,6 +249,7 @@ struct ClShared {
   int lo, hi;          // node window of the CTA's columns
   int wlo[16], whi[16];  // the windows of every CTA of the cluster
   uint32_t tmem;       // base of the CTA's tensor memory
+  int tm_m;            // the preconditioner's columns in a warp's share
   float2* gA;          // this CTA's partials as double-floats: p^T q per 5-node group,
   float4* tB;          // (r^T z, r^T r) per tile, two iterations
   Fix *fixA, *fixB, *fixR, *fixC;  // partials on the grids, of every CTA
@@ -370,9 +371,9 @@ __device__ __noinline__ Fix fix_total(const Fix* slot, int n, int lane) {
 // all poll 6,200, a mailbox per CTA that all store into 4,700, clusters of 4
 // and their mailboxes 3,700.  256 x 256 shell, us an iteration: slots 21,
 // mailboxes 15.9, this 13.6 (12.5 since K streams through registers).
-// A CTA that waits for some seconds gives up: it sets the error flag, and its
+// A CTA that waits for ten seconds gives up: it sets the error flag, and its
 // later barriers do not wait.
-constexpr int kTeamPolls = 1 << 23;  // of about 700 clocks: some seconds
+constexpr int kTeamPolls = 1 << 25;  // of about 700 clocks: ten seconds (other kernels may go first)
 constexpr int kTeamBias = 1 << 24;             // keeps the upper halves positive
 
 // The warp's share of sum k (one lane).
@@ -655,7 +656,7 @@ __global__ void __launch_bounds__(128) cluster_pack_kernel(const SysDesc* __rest
   const bool act = lane < TILE && node < S.n_nodes;
   const int j0 = act ? S.row_ptr[node] : 0, j1 = act ? S.row_ptr[node + 1] : 0;
   const int a = S.toff[t], m = S.toff[t + 1] - a;
-  float4* out = reinterpret_cast<float4*>(S.kc) + (size_t)a * CL_POS_F4 + lane;
+  float4* out = reinterpret_cast<float4*>(S.klo) + (size_t)a * CL_POS_F4 + lane;
   for (int k = 0; k < m; ++k) {
     float v[36];
 #pragma unroll
@@ -935,7 +936,7 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
   const int pa = __ldg(S.toff + ta), m = __ldg(S.toff + tb) - pa;
   if (tm_cols && w == 0) tm_alloc(&sh.tmem, tm_cols);
   __syncthreads();
-  const ulonglong2* Kg = reinterpret_cast<const ulonglong2*>(S.kc) + (size_t)pa * CL_POS_F4;
+  const ulonglong2* Kg = reinterpret_cast<const ulonglong2*>(S.klo) + (size_t)pa * CL_POS_F4;
   KPos kr[KREG ? KREG : 1];
 #pragma unroll
   for (int i = 0; i < KREG; ++i)
@@ -955,7 +956,8 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
       tm_cols ? sh.tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)((w >> 2) * tm_share) : 0u;
 #pragma unroll 1
   for (int i = 0; i < 9 * ntm; ++i) tm_st(tmw + 4 * i, __ldg(Kg + lane + 32 * i));
-  const uint32_t tmm = tmw + tm_share - tm_m;  // the preconditioner's columns
+  const uint32_t tmm = tmw + tm_share - tm_m;
+  if (tid == 0) sh.tm_m = tm_share - tm_m;
   if (m_tm)
 #pragma unroll 1
     for (int t = ta; t < tb; ++t) {
@@ -970,7 +972,7 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
   Kg += (size_t)ntm * CL_POS_F4;
 #pragma unroll 4
   for (int i = lane; i < ns * CL_POS_F4; i += 32) Kw[i] = __ldg(Kg + i);
-  Kg += (size_t)ns * CL_POS_F4;  // what streams
+  const int streamed = pa + nkr + ntm + ns;  // the first position that streams
   // the vectors of a sweep under way
   {
     const float2* r2 = reinterpret_cast<const float2*>((const float*)S.r + 6 * (size_t)n0);
@@ -1069,7 +1071,7 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
         auto row_end = [&] {
           if (--left) return;  // else the tile's rows are done
           const int l = TILE * t + lane - n0;
-          if (lane < TILE && l < nown) {
+          if (lane < TILE && l < n1 - n0) {
             float q[6];
 #pragma unroll
             for (int a = 0; a < 3; ++a) unpack2(acc[a], q[2 * a], q[2 * a + 1]);
@@ -1115,7 +1117,8 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
           __syncwarp();
         }
         if (ng > 0) {
-          const ulonglong2* kp = Kg + lane;
+          const ulonglong2* kp = reinterpret_cast<const ulonglong2*>(S.klo) +
+                                 (size_t)streamed * CL_POS_F4 + lane;
           ulonglong2 k[9];
 #pragma unroll
           for (int q = 0; q < 9; ++q) k[q] = __ldg(kp + 32 * q);
@@ -1261,7 +1264,7 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
       if (m_tm) {
         if constexpr (!JAC) {
           uint32_t r[M32_PACK];
-          tm_ld24(tmm + M32_PACK * (t - ta), r);
+          tm_ld24(tmw + sh.tm_m + M32_PACK * (t - ta), r);
           tm_wait_ld();
           tm_loaded(r);
 #pragma unroll

@@ -137,14 +137,13 @@ struct SysDesc {
   float* y;               // [6 n_agg] A_c^-1 w
   double* cdot;           // [COARSE_ROW_BLOCKS] w^T y per row block of the coarse solve
   void* zb;               // [6 n_nodes] z_b (FP32)
-  // double-float CG (precision SSO_F32X2, small.cu): the low parts of K,
-  // K64 - K32 rounded to FP32, [n_blocks * 36] (the element-block scratch)
+  // the element-block scratch.  Double-float CG (precision SSO_F32X2, small.cu):
+  // the low parts of K, K64 - K32 rounded to FP32, [n_blocks * 36].  CG on
+  // clusters (cluster.cu): K32 in that engine's layout
   float* klo;
-  // one-cluster CG (cluster.cu): block positions of the tiles [n_tiles + 1]
-  // (fixed by the mesh), K in that engine's layout (in the element-block scratch)
-  const int* toff;
-  float* kc;
   SysScalars* sc;
+  // CG on clusters: block positions of the tiles [n_tiles + 1] (fixed by the mesh)
+  const int* toff;
 };
 
 #ifdef __CUDACC__
