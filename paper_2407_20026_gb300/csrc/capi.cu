@@ -317,7 +317,8 @@ struct sso_batch {
   // SSO_F32X2: the systems being solved (one CTA each); one-cluster CG: the
   // systems by cluster size
   int* d_list = nullptr;
-  unsigned long long* d_slots = nullptr;  // CL_SLOT_BYTES: the teams' barrier words
+  // CL_SLOT_BYTES: the teams' barrier words (allocated by the first run on teams)
+  unsigned long long* d_slots = nullptr;
   std::vector<int> h_list;
   // one-cluster CG: extra streams for the launches of further cluster sizes
   cudaStream_t cl_stream[2 * CL_SIZES - 1] = {};
@@ -1435,7 +1436,10 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
                                            [](const ClusterBin& b) { return b.team; });
     for (long long launches = 1;; ++launches) {
       std::unique_lock<std::mutex> lock(g_team_mutex, std::defer_lock);
-      if (teams) lock.lock();
+      if (teams) {
+        lock.lock();
+        if (!B->d_slots) CK(cudaMalloc(&B->d_slots, CL_SLOT_BYTES));
+      }
       sso_status st = launch_bins(B, bins, B->d_list, o->precond, steps);
       if (st != SSO_OK) return st;
       for (const Team64Bin& b : bins64)
@@ -2356,7 +2360,6 @@ sso_status create_batch(sso_model* const* models, int32_t n, sso_batch** out, bo
   c.take<int>(2);
   c.take<SetupJob>(n);
   c.take<int>(n);
-  c.take<unsigned long long>(CL_SLOT_BYTES / 8);
   const size_t bytes = align_up(c.off, 256);
   std::vector<SetupJob> jobs(n);
   for (int s = 0; s < n; ++s) {
@@ -2384,7 +2387,6 @@ sso_status create_batch(sso_model* const* models, int32_t n, sso_batch** out, bo
   B->d_ccount = d.take<int>(2);
   B->d_jobs = d.take<SetupJob>(n);
   B->d_list = d.take<int>(n);
-  B->d_slots = d.take<unsigned long long>(CL_SLOT_BYTES / 8);
   B->grid_restrict = (B->n_aggs + 7) / 8;  // one warp per (system, aggregate)
   B->grid_csolve = n * COARSE_ROW_BLOCKS;  // one CTA per work item
   const int ccount[2] = {B->n_aggs, n};
@@ -2497,6 +2499,7 @@ void sso_batch_destroy(sso_batch* B) {
   }
   if (B->cl_fork) cudaEventDestroy(B->cl_fork);
   if (B->ev_fork) cudaEventDestroy(B->ev_fork);
+  if (B->d_slots) cudaFree(B->d_slots);
   if (B->arena) cudaFree(B->arena);
   if (B->h_sc) cudaFreeHost(B->h_sc);
   if (B->h_flag) cudaFreeHost(B->h_flag);
