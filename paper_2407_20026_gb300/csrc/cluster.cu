@@ -1010,6 +1010,9 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
     cl_st(cl_map(smem_addr(&sh.whi[rank]), tid), lo + wn);
   }
   if (!GRID) cl_sync();  // ... and has read the system's state and set up its windows
+  // (a launch may begin in the fold, which reads D by other threads than loaded it;
+  // nothing else separates a team's copies from its first step)
+  if (GRID) __syncthreads();
   unsigned dest = 0u;  // CTAs whose windows reach this warp's nodes
 #pragma unroll 1
   for (unsigned c = 0; !GRID && c < C; ++c)

@@ -203,3 +203,33 @@ def test_fp64_batches_launches_and_adjoint(sso, precond):
     warm = sso.Model(meshgen.gridshell(20))
     warm.solve(precision="fp64", precond=precond, rtol=1e-6)
     assert warm.solve(precision="fp64", precond=precond, rtol=1e-10, warm_start=1)["status"] == 0
+
+
+@pytest.mark.parametrize("steps", [1, 2, 3])
+def test_team_launches_begin_in_every_state(sso, steps):
+    # a team per launch of 1 to 3 steps, over several sweeps to convergence:
+    # launches begin in the first residual, the iteration, the fold and the
+    # residual after it
+    m = meshgen.gridshell(110, seed=5)
+    kw = dict(rtol=1e-6, inner_rtol=0.1, max_iter=20000)
+    want = _same(sso, [m], **kw)
+    whole = _run(sso, [m], False, **kw)
+    cut = _run(sso, [m], False, timeout_ms=1e5, iters_per_launch=steps, **kw)
+    assert want[0]["status"] == 0 and want[0]["sweeps"] > 2
+    for k in ("status", "iterations", "sweeps", "rel_residual"):
+        assert cut[0][0][k] == whole[0][0][k] == want[0][k], k
+    for k in ("u", "C", "dz", "dt", "lam"):
+        assert np.array_equal(cut[1][0][k], whole[1][0][k]), k
+
+
+def test_team_launch_that_begins_in_the_fold_at_the_cap(sso):
+    # the first launch's 1,024 steps end with the last iteration of the cap
+    m = meshgen.shell(90, seed=2)
+    kw = dict(rtol=1e-6, max_iter=1023)
+    st = _same(sso, [m], **kw)
+    assert st[0]["iterations"] == 1023 and st[0]["sweeps"] == 1
+    whole = _run(sso, [m], False, **kw)
+    for steps in (1, 2):
+        cut = _run(sso, [m], False, timeout_ms=1e5, iters_per_launch=steps, **kw)
+        assert cut[0][0]["iterations"] == whole[0][0]["iterations"]
+        assert np.array_equal(cut[1][0]["u"], whole[1][0]["u"])
