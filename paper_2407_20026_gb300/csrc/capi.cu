@@ -1248,9 +1248,74 @@ sso_status launch_bins(sso_batch* B, const std::vector<ClusterBin>& bins, const 
 }
 
 // The CTAs of a team wait for one another, so that all of them must come to
-// run: one batch at a time has teams on the device (held from a launch until
-// its completion; other kernels beside them end by themselves).
-std::mutex g_team_mutex;
+// run.  The launches with teams that are in flight on a device hold no more
+// CTAs together than it has SMs: a CTA that has not started then finds an SM
+// without another team's CTA, and kernels other than teams end by themselves.
+// A run holds its CTAs from a launch to its completion, in order of arrival.
+// (One run at a time on the device: 16 threads that each solve a 10 x 10 grid
+// shell in FP64 took 22.8 ms, two kernels an iteration 4.3.)
+struct TeamSpace {
+  std::mutex mu;
+  std::condition_variable cv;
+  int used = 0;                           // CTAs of launches in flight
+  unsigned long long ticket = 0;
+  std::deque<unsigned long long> queue;  // tickets of those that wait
+  int runs = 0;  // CG runs under way that teams or clusters may take
+};
+TeamSpace& team_space(int device) {
+  static std::mutex mu;
+  static std::map<int, TeamSpace> spaces;
+  std::lock_guard<std::mutex> lock(mu);
+  return spaces[device];
+}
+
+// n CG runs of a device, counted while this lives: each plans for its share.
+struct TeamRuns {
+  TeamSpace& space;
+  const int n;
+  TeamRuns(TeamSpace& s, int count) : space(s), n(count) {
+    std::lock_guard<std::mutex> lock(space.mu);
+    space.runs += n;
+  }
+  ~TeamRuns() {
+    std::lock_guard<std::mutex> lock(space.mu);
+    space.runs -= n;
+  }
+  static int count(TeamSpace& s) {
+    std::lock_guard<std::mutex> lock(s.mu);
+    return s.runs;
+  }
+};
+
+// CTAs of a device, held while this lives.
+struct TeamHold {
+  TeamSpace& space;
+  int n = 0;
+  explicit TeamHold(TeamSpace& s) : space(s) {}
+  // Waits for `ctas` of the device's `all`, at most to `until` (null: without
+  // limit); false: not held.
+  bool take(int ctas, int all, const std::chrono::steady_clock::time_point* until) {
+    std::unique_lock<std::mutex> lock(space.mu);
+    const unsigned long long t = space.ticket++;
+    space.queue.push_back(t);
+    auto mine = [&] { return space.queue.front() == t && space.used + ctas <= all; };
+    bool ok = true;
+    if (until)
+      ok = space.cv.wait_until(lock, *until, mine);
+    else
+      space.cv.wait(lock, mine);
+    space.queue.erase(std::find(space.queue.begin(), space.queue.end(), t));
+    if (ok) space.used += n = ctas;
+    space.cv.notify_all();
+    return ok;
+  }
+  ~TeamHold() {
+    if (!n) return;
+    std::lock_guard<std::mutex> lock(space.mu);
+    space.used -= n;
+    space.cv.notify_all();
+  }
+};
 
 // FP64 CG on teams (Jacobi and block Jacobi): one launch of systems with teams
 // of one size.
@@ -1266,10 +1331,14 @@ struct Team64Bin {
 // Measured (us an iteration of all, estimate in brackets at 1.92 GHz): one 41 x
 // 41 grid shell 11.6 (9.9), 16 of them 31.0 (28.1), 64 123 (121).  Teams were
 // faster than the two kernels at every size and count tried (10 x 10 to 100 x
-// 100, 1 to 64 systems), so that whatever fits takes them.
+// 100, 1 to 64 systems), so that whatever fits takes them.  sharers: runs of
+// about as many systems on the device at the same time, each of which takes
+// fewer CTAs (16 threads with a 41 x 41 grid shell each: 57 CTAs for one alone,
+// 8 for each of them).
 template <class GetModel>
-sso_status plan_team64(int n_sys, const std::vector<char>& active, bool jacobi, GetModel model,
-                       std::vector<int>& list, std::vector<Team64Bin>& bins, bool* fits) {
+sso_status plan_team64(int n_sys, const std::vector<char>& active, bool jacobi, int sharers,
+                       GetModel model, std::vector<int>& list, std::vector<Team64Bin>& bins,
+                       bool* fits) {
   *fits = false;
   list.clear();
   bins.clear();
@@ -1297,7 +1366,7 @@ sso_status plan_team64(int n_sys, const std::vector<char>& active, bool jacobi, 
       const bool k_in = need + k_bytes <= (size_t)dev->smem;
       const int per = std::min(dev->ctas / C, CL_MAX_TEAMS);
       const double t = 12000.0 + 7000.0 * sh.own_tiles + (k_in ? 0.0 : k_bytes / 64.0);
-      const double all = t * ((n_act + per - 1) / per);
+      const double all = t * ((n_act * (long long)sharers + per - 1) / per);
       if (all < best_t) {
         best_t = all;
         best = {s, C, std::min(TEAM64_THREADS, 32 * WARPS * sh.own_tiles),
@@ -1328,6 +1397,9 @@ sso_status plan_team64(int n_sys, const std::vector<char>& active, bool jacobi, 
 // microseconds) does not count, short enough that the host sees finished
 // systems and the wall-clock cap within a few milliseconds.
 constexpr int kClusterSteps = 1024;
+// ... with teams, while other runs of the device wait for its SMs (a launch's
+// own time is about 30 us: 1 % of these).
+constexpr int kSharedSteps = 256;
 
 // defer: return after queuing the copy of the scalars, without waiting (the
 // caller synchronises the stream and calls finish_run).
@@ -1350,13 +1422,15 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
   bool cluster = false;
   std::vector<ClusterBin> bins;
   std::vector<Team64Bin> bins64;
+  TeamSpace& space = team_space(B->models[0]->device);
+  const int sharers = std::max(1, TeamRuns::count(space));
   if (o->precision == SSO_FP32_IR && !B->profiling) {
-    sso_status st = plan_bins(B->n_sys, active, o->precond, 1, true,
+    sso_status st = plan_bins(B->n_sys, active, o->precond, sharers, true,
                               [B](int s) { return B->models[s]; }, B->h_list, bins, &cluster);
     if (st != SSO_OK) return st;
   }
   if (fp64 && !B->profiling && (o->precond == SSO_JACOBI || o->precond == SSO_BLOCK_JACOBI)) {
-    sso_status st = plan_team64(B->n_sys, active, o->precond == SSO_JACOBI,
+    sso_status st = plan_team64(B->n_sys, active, o->precond == SSO_JACOBI, sharers,
                                 [B](int s) { return B->models[s]; }, B->h_list, bins64, &cluster);
     if (st != SSO_OK) return st;
   }
@@ -1431,21 +1505,43 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
          1);
     const int steps = o->timeout_ms > 0.0 ? std::min(kClusterSteps, o->iters_per_launch)
                                           : kClusterSteps;
-    const long long max_launches = (2LL * o->max_iter + 4LL * o->max_sweeps) / steps + 8;
-    const bool teams = fp64 || std::any_of(bins.begin(), bins.end(),
-                                           [](const ClusterBin& b) { return b.team; });
+    const long long max_launches =
+        (2LL * o->max_iter + 4LL * o->max_sweeps) / std::min(steps, kSharedSteps) + 8;
+    const ClusterDevice* dev = nullptr;
+    sso_status st = cluster_device(&dev);
+    if (st != SSO_OK) return st;
+    int ctas = 0;  // of the largest launch with teams
+    for (const ClusterBin& b : bins)
+      if (b.team)
+        ctas = std::max(ctas, b.size * std::min(b.n, std::min(dev->ctas / b.size, CL_MAX_TEAMS)));
+    for (const Team64Bin& b : bins64) ctas = std::max(ctas, b.team * b.n);
+    if (ctas && !B->d_slots) CK(cudaMalloc(&B->d_slots, CL_SLOT_BYTES));
+    const auto until = t0 + std::chrono::duration_cast<std::chrono::steady_clock::duration>(
+                                std::chrono::duration<double, std::milli>(
+                                    std::min(std::max(o->timeout_ms, 0.0), 1e12)));
     for (long long launches = 1;; ++launches) {
-      std::unique_lock<std::mutex> lock(g_team_mutex, std::defer_lock);
-      if (teams) {
-        lock.lock();
-        if (!B->d_slots) CK(cudaMalloc(&B->d_slots, CL_SLOT_BYTES));
+      TeamHold hold(space);
+      int now = steps;
+      if (ctas) {
+        // (the first launch waits for its turn whatever the wall-clock cap, so
+        // that a run always has a residual to report)
+        if (!hold.take(ctas, dev->ctas, launches > 1 && o->timeout_ms > 0.0 ? &until : nullptr))
+          break;
+        if (TeamRuns::count(space) > 1) now = std::min(steps, kSharedSteps);
       }
-      sso_status st = launch_bins(B, bins, B->d_list, o->precond, steps);
-      if (st != SSO_OK) return st;
-      for (const Team64Bin& b : bins64)
-        CL(launch_team64(B->d_sys, B->d_list + b.first, b.n, b.team, b.threads, b.smem,
-                         o->precond == SSO_JACOBI, B->d_slots, B->d_n_active, steps, B->stream),
-           1);
+      st = launch_bins(B, bins, B->d_list, o->precond, now);
+      for (size_t i = 0; i < bins64.size() && st == SSO_OK; ++i) {
+        const Team64Bin& b = bins64[i];
+        const cudaError_t e =
+            launch_team64(B->d_sys, B->d_list + b.first, b.n, b.team, b.threads, b.smem,
+                          o->precond == SSO_JACOBI, B->d_slots, B->d_n_active, now, B->stream);
+        g_launches += 1;
+        if (e != cudaSuccess) st = cuda_fail(e, "launch_team64");
+      }
+      if (st != SSO_OK) {
+        cudaStreamSynchronize(B->stream);  // teams under way still hold their CTAs
+        return st;
+      }
       CK(cudaMemcpyAsync(B->h_flag + 2, B->d_n_active, 2 * sizeof(int), cudaMemcpyDeviceToHost,
                          B->stream));
       CK(cudaEventRecord(B->ev, B->stream));
@@ -1563,7 +1659,12 @@ sso_status finish_run(sso_batch* B, const std::vector<char>& active, sso_stats* 
 // the work already on the batch's stream, which then waits for them.
 sso_status run_cg(sso_batch* B, const sso_options* o, bool adjoint,
                   const std::vector<char>& active, sso_stats* stats, bool* deferred = nullptr) {
-  if (B->parts.empty() || B->profiling) {
+  const bool whole = B->parts.empty() || B->profiling;
+  const TeamRuns runs(team_space(B->models[0]->device),
+                      o->precision == SSO_F32X2 || o->precond == SSO_CHAIN || B->profiling ? 0
+                      : whole                                                             ? 1
+                                              : (int)B->parts.size());
+  if (whole) {
     // one launch and no host loop (double-float CG): the caller may fold
     // the wait for it into its own
     const bool defer = deferred && o->precision == SSO_F32X2 && o->precond != SSO_CHAIN;
@@ -1577,6 +1678,7 @@ sso_status run_cg(sso_batch* B, const sso_options* o, bool adjoint,
   std::vector<sso_status> res(np, SSO_OK);
   std::vector<std::string> msg(np);
   auto work = [&](int k) {
+    cudaSetDevice(B->models[0]->device);  // (the threads' own)
     const std::vector<char> act(active.begin() + B->part0[k], active.begin() + B->part0[k + 1]);
     res[k] = batch_run(B->parts[k], o, adjoint, act, stats ? stats + B->part0[k] : nullptr);
     if (res[k] != SSO_OK) msg[k] = g_last_error;

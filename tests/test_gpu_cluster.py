@@ -233,3 +233,35 @@ def test_team_launch_that_begins_in_the_fold_at_the_cap(sso):
         cut = _run(sso, [m], False, timeout_ms=1e5, iters_per_launch=steps, **kw)
         assert cut[0][0]["iterations"] == whole[0][0]["iterations"]
         assert np.array_equal(cut[1][0]["u"], whole[1][0]["u"])
+
+
+def test_teams_of_several_threads_and_parts(sso):
+    # solves with teams at the same time (each plans for its share of the SMs)
+    # give the bits of each solve alone
+    import threading
+    cases = [(meshgen.gridshell(10, seed=1), dict(precision="fp64", rtol=1e-10)),
+             (meshgen.gridshell(41, seed=2), dict(precision="fp64", rtol=1e-10)),
+             (meshgen.gridshell(100, seed=3), dict(precision="fp64", rtol=1e-10, max_iter=400)),
+             (meshgen.shell(90, seed=4), dict(rtol=1e-6, max_iter=600)),
+             (meshgen.gridshell(110, seed=5), dict(rtol=1e-6, max_iter=600)),
+             (meshgen.shell(30, seed=6), dict(rtol=1e-6, max_iter=600))] * 2
+    want = [_run(sso, [m], True, **kw) for m, kw in cases]
+    models = [sso.Model(m) for m, _ in cases]
+    got = [None] * len(cases)
+
+    def work(i):
+        for _ in range(3):
+            st = models[i].solve(sso.options(**cases[i][1]), raise_on_error=False)
+            got[i] = (st, models[i].result())
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(len(cases))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for (st, res), (wst, wres) in zip(got, want):
+        assert (st["status"], st["iterations"]) == (wst[0]["status"], wst[0]["iterations"])
+        assert np.array_equal(res["u"], wres[0]["u"])
+    # 32 models and more run as parts on threads of their own
+    _same(sso, [meshgen.gridshell(9 + k % 3, seed=k) for k in range(34)], precision="fp64",
+          rtol=1e-10)
+    _same(sso, [meshgen.gridshell(110, seed=k) for k in range(32)], rtol=1e-6, max_iter=60)
