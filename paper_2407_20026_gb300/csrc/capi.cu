@@ -1317,79 +1317,155 @@ struct TeamHold {
   }
 };
 
-// FP64 CG on teams (Jacobi and block Jacobi): one launch of systems with teams
-// of one size.
+// FP64 CG on teams (Jacobi and block Jacobi): one launch of `n` systems, listed
+// from entry `first` on and followed there by their n + 1 first CTAs.
 struct Team64Bin {
-  int first, n, team, threads, smem;
+  int first, n, ctas, threads, smem;
 };
 
-// Sorts the active systems into launches; *fits is false when one does not fit
-// (the batch then runs the two-kernel engine).  Tiles per CTA by the least
-// estimated time of all: an iteration is the barriers and sums (12,000 clocks),
-// plus the FP64 pipe's work on a tile (7,000) and K from L2 where it does not
-// fit shared memory; systems beyond those resident at once run in waves.
-// Measured (us an iteration of all, estimate in brackets at 1.92 GHz): one 41 x
-// 41 grid shell 11.6 (9.9), 16 of them 31.0 (28.1), 64 123 (121).  Teams were
-// faster than the two kernels at every size and count tried (10 x 10 to 100 x
-// 100, 1 to 64 systems), so that whatever fits takes them.  sharers: runs of
-// about as many systems on the device at the same time, each of which takes
-// fewer CTAs (16 threads with a 41 x 41 grid shell each: 57 CTAs for one alone,
-// 8 for each of them).
+// A system's team: its CTAs and the estimated clocks of an iteration, the
+// barriers (12,000; one CTA: 8,000), the sums of the tiles' partials, the FP64 pipe's work on the
+// blocks of a CTA and K from L2 where it does not fit shared memory.
+// Measured (clocks of an iteration at 1.92 GHz, estimate in brackets): one 41 x
+// 41 grid shell on 57 CTAs 22,000 (19,000), 4 of 100 x 100 on 38 each 77,000
+// (81,000), one of 190 x 190 on 151 91,000 (85,000).
+struct Team64Share {
+  int sys, ctas, threads, smem;
+  double clocks;
+};
+// With `tiles` tiles a CTA, or as near to that as fits; false: none fits.
+bool team64_share(const sso_model* M, bool jacobi, int tiles, const ClusterDevice& d,
+                  Team64Share* out) {
+  for (int i = 0; i < TEAM64_TILES; ++i) {
+    // tiles, tiles + 1, ... and then tiles - 1, tiles - 2, ...
+    const int k = tiles - 1 + i < TEAM64_TILES ? tiles - 1 + i : TEAM64_TILES - 1 - i;
+    const ClusterShare& sh = M->cl_team64[k];
+    const int C = (M->n_tiles + k) / (k + 1);
+    if (!sh.n_tiles || C > d.ctas) continue;
+    size_t k_bytes = 0;
+    const size_t need = team64_smem_bytes(sh, jacobi, &k_bytes);
+    if (need > (size_t)d.smem) continue;
+    const bool k_in = need + k_bytes <= (size_t)d.smem;
+    out->ctas = C;
+    out->threads = std::min(TEAM64_THREADS, 32 * WARPS * sh.own_tiles);
+    out->smem = (int)(need + (k_in ? k_bytes : 0));
+    out->clocks = (C > 1 ? 12000.0 : 8000.0) + 12.5 * M->n_tiles + 2000.0 * sh.own_tiles + 20.0 * sh.members +
+                  (k_in ? 0.0 : k_bytes / 64.0);
+    return true;
+  }
+  return false;
+}
+
+// The two kernels' clocks of an iteration of a system's blocks, beside 42,000 for
+// the launches and sums of an iteration of all systems.  Measured: 64 41 x 41
+// grid shells 257,000 (estimate 280,000), 4 of 100 x 100 170,000 (160,000), 1,024
+// of 10 x 10 290,000 (310,000).
+double two64_clocks(const sso_model* M) {
+  return 100.0 + M->n_blocks * (0.29 + 0.14 * std::min(1.0, M->n_tiles / 330.0));
+}
+// Runs whose work the device takes at once, however little it is (a device has
+// 8 hardware queues unless the environment says otherwise).
+constexpr int kTeamQueues = 8;
+// Teams where their estimate times a margin is better, as launches of teams wait
+// for the last of their systems, and teams of several runs for one another.
+// Measured, two kernels -> teams: 256 10 x 10 grid shells 12.8 -> 10.2 ms, 32 of
+// sides 8 to 60 71 -> 40, 256 of 41 x 41 173 -> 137; solves of 8 threads at
+// once, 41 x 41 18.0 -> 12.8, 100 x 100 62 -> 45, of 16, 100 x 100 130 -> 90; and
+// not taken, 16 threads with 41 x 41 21.5 -> 24.5.
+constexpr double kTeam64Margin = 1.08;
+double team64_margin(int sharers, int together) {
+  return sharers == 1 ? kTeam64Margin : 1.0 + 0.1 * together;
+}
+
+// Sorts the active systems into launches of teams of any sizes; *fits is false
+// when one does not fit or the two kernels should be faster (`compare`).  All
+// systems take about the same number of tiles a CTA, the one of the least
+// estimated time for all launches, one after another.  sharers: runs of about
+// as many systems on the device at the same time, each of which takes fewer
+// CTAs (8 threads with a 41 x 41 grid shell each: 57 CTAs for one alone, 15 for
+// each of them).
 template <class GetModel>
 sso_status plan_team64(int n_sys, const std::vector<char>& active, bool jacobi, int sharers,
-                       GetModel model, std::vector<int>& list, std::vector<Team64Bin>& bins,
-                       bool* fits) {
+                       bool compare, GetModel model, std::vector<int>& list,
+                       std::vector<Team64Bin>& bins, bool* fits) {
   *fits = false;
   list.clear();
   bins.clear();
   const ClusterDevice* dev = nullptr;
   sso_status st = cluster_device(&dev);
   if (st != SSO_OK) return st;
-  int n_act = 0;
-  for (int s = 0; s < n_sys; ++s) n_act += active[s] != 0;
-  struct Choice {
-    int sys, team, threads, smem;
+  struct Launch {
+    int ctas = 0;
+    double clocks = 0.0;
+    std::vector<int> shares;
   };
-  std::vector<Choice> choice;
-  for (int s = 0; s < n_sys; ++s) {
-    if (!active[s]) continue;
-    const sso_model* M = model(s);
-    Choice best{s, 0, 0, 0};
-    double best_t = HUGE_VAL;
-    for (int k = 0; k < TEAM64_TILES; ++k) {
-      const ClusterShare& sh = M->cl_team64[k];
-      const int C = (M->n_tiles + k) / (k + 1);
-      if (!sh.n_tiles || C > dev->ctas) continue;
-      size_t k_bytes = 0;
-      const size_t need = team64_smem_bytes(sh, jacobi, &k_bytes);
-      if (need > (size_t)dev->smem) continue;
-      const bool k_in = need + k_bytes <= (size_t)dev->smem;
-      const int per = std::min(dev->ctas / C, CL_MAX_TEAMS);
-      const double t = 12000.0 + 7000.0 * sh.own_tiles + (k_in ? 0.0 : k_bytes / 64.0);
-      const double all = t * ((n_act * (long long)sharers + per - 1) / per);
-      if (all < best_t) {
-        best_t = all;
-        best = {s, C, std::min(TEAM64_THREADS, 32 * WARPS * sh.own_tiles),
-                (int)(need + (k_in ? k_bytes : 0))};
-      }
+  std::vector<Team64Share> shares, sorted, best_shares;
+  std::vector<Launch> best;
+  double best_t = HUGE_VAL, two = 0.0;
+  for (int s = 0; s < n_sys; ++s)
+    if (active[s]) two += sharers * two64_clocks(model(s));
+  for (int k = 1; k <= TEAM64_TILES; ++k) {
+    shares.clear();
+    for (int s = 0; s < n_sys; ++s) {
+      if (!active[s]) continue;
+      Team64Share h{s, 0, 0, 0, 0.0};
+      if (!team64_share(model(s), jacobi, k, *dev, &h)) return SSO_OK;
+      shares.push_back(h);
     }
-    if (!best.team) return SSO_OK;
-    choice.push_back(best);
+    {  // the largest teams first
+      std::vector<int> at(dev->ctas + 2, 0);
+      for (const Team64Share& h : shares) ++at[dev->ctas - h.ctas + 1];
+      for (int c = 0; c <= dev->ctas; ++c) at[c + 1] += at[c];
+      sorted.resize(shares.size());
+      for (const Team64Share& h : shares) sorted[at[dev->ctas - h.ctas]++] = h;
+      shares.swap(sorted);
+    }
+    std::vector<Launch> launches;
+    size_t open = 0;  // the first launch that the smallest team still fits
+    for (int i = 0; i < (int)shares.size(); ++i) {
+      const int C = shares[i].ctas;
+      while (open < launches.size() &&
+             (launches[open].ctas + shares.back().ctas > dev->ctas ||
+              (int)launches[open].shares.size() == CL_MAX_TEAMS))
+        ++open;
+      size_t at = open;
+      while (at < launches.size() && (launches[at].ctas + C > dev->ctas ||
+                                      (int)launches[at].shares.size() == CL_MAX_TEAMS))
+        ++at;
+      if (at == launches.size()) launches.emplace_back();
+      Launch& l = launches[at];
+      l.ctas += C;
+      l.clocks = std::max(l.clocks, shares[i].clocks);
+      l.shares.push_back(i);
+    }
+    double t = 0.0;
+    for (const Launch& l : launches) {
+      const int together = std::min(kTeamQueues, std::max(1, dev->ctas / l.ctas));
+      t += l.clocks * std::max(1.0, (double)sharers / together) * team64_margin(sharers, together);
+    }
+    if (t < best_t) {
+      best_t = t;
+      best.swap(launches);
+      best_shares.swap(shares);
+    }
   }
-  std::stable_sort(choice.begin(), choice.end(),
-                   [](const Choice& a, const Choice& b) { return a.team > b.team; });
-  for (size_t i = 0; i < choice.size(); ++i) {
-    const Choice& c = choice[i];
-    const int per = std::min(dev->ctas / c.team, CL_MAX_TEAMS);
-    if (bins.empty() || bins.back().team != c.team || bins.back().n == per)
-      bins.push_back({(int)i, 0, c.team, 0, 0});
-    Team64Bin& b = bins.back();
-    ++b.n;
-    b.threads = std::max(b.threads, c.threads);
-    b.smem = std::max(b.smem, c.smem);
-    list.push_back(c.sys);
+  const double launches_two = 42000.0 * sharers / kTeamQueues;
+  if (best.empty() || (compare && best_t > std::max(launches_two, 42000.0 + two))) return SSO_OK;
+  for (const Launch& l : best) {
+    Team64Bin b{(int)list.size(), (int)l.shares.size(), l.ctas, 0, 0};
+    for (int i : l.shares) list.push_back(best_shares[i].sys);
+    int at = 0;
+    for (int i : l.shares) {
+      const Team64Share& h = best_shares[i];
+      list.push_back(at);
+      at += h.ctas;
+      b.threads = std::max(b.threads, h.threads);
+      b.smem = std::max(b.smem, h.smem);
+    }
+    list.push_back(at);
+    bins.push_back(b);
   }
-  *fits = !list.empty();
+  *fits = true;
   return SSO_OK;
 }
 
@@ -1397,14 +1473,24 @@ sso_status plan_team64(int n_sys, const std::vector<char>& active, bool jacobi, 
 // microseconds) does not count, short enough that the host sees finished
 // systems and the wall-clock cap within a few milliseconds.
 constexpr int kClusterSteps = 1024;
-// ... with teams, while other runs of the device wait for its SMs (a launch's
-// own time is about 30 us: 1 % of these).
+// ... with teams, while other runs of the device wait for its SMs, and of
+// several systems in FP64, whose launches are planned again for those that have
+// not finished (a launch's own time is about 30 us: 1 % of these).
 constexpr int kSharedSteps = 256;
 
+// FP64 runs that may take teams.
+bool team64_options(const sso_options* o) {
+  return o->precision == SSO_FP64 &&
+         (o->precond == SSO_JACOBI || o->precond == SSO_BLOCK_JACOBI);
+}
+
 // defer: return after queuing the copy of the scalars, without waiting (the
-// caller synchronises the stream and calls finish_run).
+// caller synchronises the stream and calls finish_run).  plan: the launches of
+// teams that the caller has planned into B's list for an FP64 run (empty: two
+// kernels); without it the run plans for itself.
 sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
-                     const std::vector<char>& active, sso_stats* stats, bool defer = false) {
+                     const std::vector<char>& active, sso_stats* stats, bool defer = false,
+                     const std::vector<Team64Bin>* plan = nullptr) {
   if (o->precond == SSO_CHAIN) return chain_run(B, o, adjoint, active, stats);
   const auto t0 = std::chrono::steady_clock::now();
   const bool fp64 = o->precision == SSO_FP64;
@@ -1429,9 +1515,16 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
                               [B](int s) { return B->models[s]; }, B->h_list, bins, &cluster);
     if (st != SSO_OK) return st;
   }
-  if (fp64 && !B->profiling && (o->precond == SSO_JACOBI || o->precond == SSO_BLOCK_JACOBI)) {
-    sso_status st = plan_team64(B->n_sys, active, o->precond == SSO_JACOBI, sharers,
-                                [B](int s) { return B->models[s]; }, B->h_list, bins64, &cluster);
+  auto plan64 = [&](const std::vector<char>& systems, bool compare, bool* fits) {
+    return plan_team64(B->n_sys, systems, o->precond == SSO_JACOBI,
+                       std::max(1, TeamRuns::count(space)), compare,
+                       [B](int s) { return B->models[s]; }, B->h_list, bins64, fits);
+  };
+  if (plan) {
+    bins64 = *plan;
+    cluster = !plan->empty();
+  } else if (team64_options(o) && !B->profiling) {
+    sso_status st = plan64(active, true, &cluster);
     if (st != SSO_OK) return st;
   }
   int n_act = 0;
@@ -1498,23 +1591,24 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
   } else if (n_act > 0 && cluster) {
     CK(cudaMemcpyAsync(B->d_list, B->h_list.data(), B->h_list.size() * sizeof(int),
                        cudaMemcpyHostToDevice, B->stream));
-    int max_nodes = 1;
-    for (int s : B->h_list) max_nodes = std::max(max_nodes, B->models[s]->n_nodes);
-    if (!fp64)
+    if (!fp64) {
+      int max_nodes = 1;
+      for (int s : B->h_list) max_nodes = std::max(max_nodes, B->models[s]->n_nodes);
       CL(launch_cluster_pack(B->d_sys, B->d_list, (int)B->h_list.size(), max_nodes, B->stream),
          1);
-    const int steps = o->timeout_ms > 0.0 ? std::min(kClusterSteps, o->iters_per_launch)
-                                          : kClusterSteps;
+    }
+    const int most = fp64 && n_act > 1 ? kSharedSteps : kClusterSteps;
+    const int steps = o->timeout_ms > 0.0 ? std::min(most, o->iters_per_launch) : most;
     const long long max_launches =
         (2LL * o->max_iter + 4LL * o->max_sweeps) / std::min(steps, kSharedSteps) + 8;
     const ClusterDevice* dev = nullptr;
     sso_status st = cluster_device(&dev);
     if (st != SSO_OK) return st;
-    int ctas = 0;  // of the largest launch with teams
+    int ctas = 0, n_left = n_act;  // CTAs of the largest launch with teams; systems under way
     for (const ClusterBin& b : bins)
       if (b.team)
         ctas = std::max(ctas, b.size * std::min(b.n, std::min(dev->ctas / b.size, CL_MAX_TEAMS)));
-    for (const Team64Bin& b : bins64) ctas = std::max(ctas, b.team * b.n);
+    for (const Team64Bin& b : bins64) ctas = std::max(ctas, b.ctas);
     if (ctas && !B->d_slots) CK(cudaMalloc(&B->d_slots, CL_SLOT_BYTES));
     const auto until = t0 + std::chrono::duration_cast<std::chrono::steady_clock::duration>(
                                 std::chrono::duration<double, std::milli>(
@@ -1533,7 +1627,7 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
       for (size_t i = 0; i < bins64.size() && st == SSO_OK; ++i) {
         const Team64Bin& b = bins64[i];
         const cudaError_t e =
-            launch_team64(B->d_sys, B->d_list + b.first, b.n, b.team, b.threads, b.smem,
+            launch_team64(B->d_sys, B->d_list + b.first, b.n, b.ctas, b.threads, b.smem,
                           o->precond == SSO_JACOBI, B->d_slots, B->d_n_active, now, B->stream);
         g_launches += 1;
         if (e != cudaSuccess) st = cuda_fail(e, "launch_team64");
@@ -1553,6 +1647,20 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
                                      std::chrono::steady_clock::now() - t0).count() >
                                      o->timeout_ms)
         break;
+      if (!bins64.empty() && B->h_flag[2] < n_left) {  // plan for those left
+        n_left = B->h_flag[2];
+        CK(cudaMemcpyAsync(B->h_sc, B->d_sc, sizeof(SysScalars) * B->n_sys,
+                           cudaMemcpyDeviceToHost, B->stream));
+        CK(cudaStreamSynchronize(B->stream));
+        std::vector<char> left(B->n_sys);
+        for (int s = 0; s < B->n_sys; ++s) left[s] = B->h_sc[s].state != ST_DONE;
+        bool fits = false;
+        if ((st = plan64(left, false, &fits)) != SSO_OK) return st;
+        CK(cudaMemcpyAsync(B->d_list, B->h_list.data(), B->h_list.size() * sizeof(int),
+                           cudaMemcpyHostToDevice, B->stream));
+        ctas = 0;
+        for (const Team64Bin& b : bins64) ctas = std::max(ctas, b.ctas);
+      }
     }
   } else if (n_act > 0) {
     const bool two_level = o->precond == SSO_TWO_LEVEL;
@@ -1659,17 +1767,26 @@ sso_status finish_run(sso_batch* B, const std::vector<char>& active, sso_stats* 
 // the work already on the batch's stream, which then waits for them.
 sso_status run_cg(sso_batch* B, const sso_options* o, bool adjoint,
                   const std::vector<char>& active, sso_stats* stats, bool* deferred = nullptr) {
-  const bool whole = B->parts.empty() || B->profiling;
-  const TeamRuns runs(team_space(B->models[0]->device),
-                      o->precision == SSO_F32X2 || o->precond == SSO_CHAIN || B->profiling ? 0
-                      : whole                                                             ? 1
-                                              : (int)B->parts.size());
+  bool whole = B->parts.empty() || B->profiling;
+  std::vector<Team64Bin> bins64;
+  const std::vector<Team64Bin>* plan = nullptr;
+  TeamSpace& space = team_space(B->models[0]->device);
+  if (!whole && team64_options(o)) {  // teams of the whole batch, or the parts' two kernels
+    sso_status st = plan_team64(B->n_sys, active, o->precond == SSO_JACOBI,
+                                1 + TeamRuns::count(space), true,
+                                [B](int s) { return B->models[s]; }, B->h_list, bins64, &whole);
+    if (st != SSO_OK) return st;
+    plan = &bins64;
+  }
+  const TeamRuns runs(space, o->precision == SSO_F32X2 || o->precond == SSO_CHAIN || B->profiling ? 0
+                             : whole                                                             ? 1
+                                                     : (int)B->parts.size());
   if (whole) {
     // one launch and no host loop (double-float CG): the caller may fold
     // the wait for it into its own
     const bool defer = deferred && o->precision == SSO_F32X2 && o->precond != SSO_CHAIN;
     if (deferred) *deferred = defer;
-    return batch_run(B, o, adjoint, active, stats, defer);
+    return batch_run(B, o, adjoint, active, stats, defer, plan);
   }
   if (deferred) *deferred = false;
   const int np = (int)B->parts.size();
@@ -1680,7 +1797,8 @@ sso_status run_cg(sso_batch* B, const sso_options* o, bool adjoint,
   auto work = [&](int k) {
     cudaSetDevice(B->models[0]->device);  // (the threads' own)
     const std::vector<char> act(active.begin() + B->part0[k], active.begin() + B->part0[k + 1]);
-    res[k] = batch_run(B->parts[k], o, adjoint, act, stats ? stats + B->part0[k] : nullptr);
+    res[k] = batch_run(B->parts[k], o, adjoint, act, stats ? stats + B->part0[k] : nullptr, false,
+                       plan);
     if (res[k] != SSO_OK) msg[k] = g_last_error;
   };
   std::vector<std::thread> threads;
@@ -1769,16 +1887,21 @@ void plan_cluster(sso_model* M, const HostTopo& T) {
   M->cl_positions = T.toff[M->n_tiles];
   const size_t room = (size_t)std::max(M->n_eb, M->n_blocks) * 36 * sizeof(double);
   M->cluster_ok = n_chunks_of(M) <= CL_MAX_CHUNKS && cluster_pack_bytes(M) <= room;
+  std::vector<int> tlo(M->n_tiles, n), thi(M->n_tiles, 0);  // nodes that a tile's rows read
+  for (int i = 0; i < n; ++i) {
+    int &lo = tlo[i / TILE], &hi = thi[i / TILE];
+    lo = std::min(lo, T.col[T.row_ptr[i]]);
+    hi = std::max(hi, T.col[T.row_ptr[i + 1] - 1] + 1);
+  }
   auto share = [&](int C) {
     int win = 0, pos = 0;
     for (int r = 0; r < C; ++r) {  // the kernel's split of the tiles
       const int t0 = (int)((long long)M->n_tiles * r / C);
       const int t1 = (int)((long long)M->n_tiles * (r + 1) / C);
-      const int n0 = std::min(n, TILE * t0), n1 = std::min(n, TILE * t1);
       int lo = n, hi = 0;
-      for (int i = n0; i < n1; ++i) {
-        lo = std::min(lo, T.col[T.row_ptr[i]]);
-        hi = std::max(hi, T.col[T.row_ptr[i + 1] - 1] + 1);
+      for (int t = t0; t < t1; ++t) {
+        lo = std::min(lo, tlo[t]);
+        hi = std::max(hi, thi[t]);
       }
       if (hi > lo) win = std::max(win, hi - lo);
       pos = std::max(pos, T.toff[t1] - T.toff[t0]);
@@ -2461,7 +2584,7 @@ sso_status create_batch(sso_model* const* models, int32_t n, sso_batch** out, bo
   c.take<int>(n);
   c.take<int>(2);
   c.take<SetupJob>(n);
-  c.take<int>(n);
+  c.take<int>(3 * (size_t)n);
   const size_t bytes = align_up(c.off, 256);
   std::vector<SetupJob> jobs(n);
   for (int s = 0; s < n; ++s) {
@@ -2488,7 +2611,7 @@ sso_status create_batch(sso_model* const* models, int32_t n, sso_batch** out, bo
   B->d_csys = d.take<int>(n);
   B->d_ccount = d.take<int>(2);
   B->d_jobs = d.take<SetupJob>(n);
-  B->d_list = d.take<int>(n);
+  B->d_list = d.take<int>(3 * (size_t)n);  // (FP64 teams: with first CTAs, a sentinel a launch)
   B->grid_restrict = (B->n_aggs + 7) / 8;  // one warp per (system, aggregate)
   B->grid_csolve = n * COARSE_ROW_BLOCKS;  // one CTA per work item
   const int ccount[2] = {B->n_aggs, n};

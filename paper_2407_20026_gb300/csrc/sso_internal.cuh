@@ -516,7 +516,7 @@ constexpr int cl_team_of(int k) {
   constexpr int size[CL_TEAMS] = {152, 76, 38};
   return size[k];
 }
-constexpr int CL_MAX_TEAMS = 16;  // of a launch
+constexpr int CL_MAX_TEAMS = 152;  // of a launch (FP64: of a CTA each)
 // a team's barrier words: two sets of lines of 128 bytes
 constexpr int CL_TEAM_COPIES = 10, CL_TEAM_WORDS = 2 * CL_TEAM_COPIES * 16;
 constexpr size_t CL_SLOT_BYTES = 8 * (size_t)CL_TEAM_WORDS * CL_MAX_TEAMS;
@@ -545,10 +545,11 @@ struct ClusterShare {
 size_t cluster_smem_bytes(const ClusterShare& c, int precond, bool m_tm, bool team);
 int cluster_tm_positions(int smem, int own_tiles, int warps, bool m_tm);
 // The FP64 CG on teams: CTAs of one to TEAM64_TILES tiles each, six warps a
-// tile.  Its ClusterShare's members are the blocks of a CTA's rows.
-constexpr int TEAM64_THREADS = 384, TEAM64_TILES = 8;
+// tile.  Its ClusterShare's members are the blocks of a CTA's rows.  A launch of
+// `ctas` CTAs runs n_list systems: list holds them, then n_list + 1 first CTAs.
+constexpr int TEAM64_THREADS = 384, TEAM64_TILES = 12;
 size_t team64_smem_bytes(const ClusterShare& c, bool jacobi, size_t* k_bytes);
-cudaError_t launch_team64(const SysDesc* sys, const int* list, int n_list, int team, int threads,
+cudaError_t launch_team64(const SysDesc* sys, const int* list, int n_list, int ctas, int threads,
                           int smem, bool jacobi, unsigned long long* slots, int* flags,
                           int max_steps, cudaStream_t s);
 // The dynamic shared memory of a CTA and the clusters of each size that are

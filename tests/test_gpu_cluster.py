@@ -265,3 +265,18 @@ def test_teams_of_several_threads_and_parts(sso):
     _same(sso, [meshgen.gridshell(9 + k % 3, seed=k) for k in range(34)], precision="fp64",
           rtol=1e-10)
     _same(sso, [meshgen.gridshell(110, seed=k) for k in range(32)], rtol=1e-6, max_iter=60)
+
+
+@pytest.mark.parametrize("precond", ["jacobi", "block_jacobi"])
+def test_fp64_batches_of_unequal_and_many_systems(sso, precond):
+    # teams of different sizes in a launch, of one CTA, more systems than a
+    # launch takes, launches planned again as systems finish, a split batch
+    kw = dict(precision="fp64", precond=precond, rtol=1e-10, max_iter=1500)
+    sides = [8, 13, 19, 24, 30, 41, 52, 60]
+    _same(sso, [meshgen.gridshell(s, seed=s) for s in sides] + [_strip(2), meshgen.shell(24)], **kw)
+    many = [meshgen.gridshell(6 + k % 5, seed=k) for k in range(170)]
+    _same(sso, many + [meshgen.gridshell(41, seed=1)], **kw)
+    g = np.random.default_rng(4)
+    meshes = [meshgen.gridshell(7 + 2 * k, seed=k) for k in range(12)]
+    _same(sso, meshes, g=[g.standard_normal(6 * m["xyz"].shape[0]) * (k % 3 == 0)
+                          for k, m in enumerate(meshes)], **kw)
