@@ -125,7 +125,8 @@ typedef struct {
   int32_t max_sweeps;        /* cap on refinement sweeps (FP64 residual recomputations) */
   int32_t iters_per_launch;  /* CG iterations per captured CUDA-graph launch; engines that keep
                                 a system on chip make up to 1024 a launch (with timeout_ms:
-                                no more than iters_per_launch; in a server: four times it) */
+                                no more than iters_per_launch; in a server: four times it;
+                                FP32 launches of less than 4, two-level 10, take the graph) */
   int32_t warm_start;        /* 1: start from the model's current u instead of 0 */
   double timeout_ms;         /* wall-clock cap, <= 0 for none */
 } sso_options;

@@ -1478,6 +1478,16 @@ constexpr int kClusterSteps = 1024;
 // not finished (a launch's own time is about 30 us: 1 % of these).
 constexpr int kSharedSteps = 256;
 
+// Whether launches of `steps` steps pay on clusters and teams in FP32, which load
+// a system's K, preconditioner and vectors in every launch: two kernels -> here
+// with a wall-clock cap, 64 x 64 shell, ms: 1 step 7.5 -> 10.1, 2 5.2 -> 6.4, 4
+// 4.6 -> 4.1, 8 4.1 -> 2.9; 48 of them 22 -> 40, 20 -> 26, 19.4 -> 17.8, 19.1 ->
+// 14.1; two-level, one 2 steps 7.9 -> 16.7, 8 6.8 -> 6.6, 12 6.7 -> 5.2, 48 8 26.1
+// -> 27.6, 12 26.0 -> 23.5.  (FP64 teams: 1 step 10.3 -> 10.0, 2 9.1 -> 6.7.)
+bool cluster_pays(int steps, int precond) {
+  return steps >= (precond == SSO_TWO_LEVEL ? 10 : 4);
+}
+
 // FP64 runs that may take teams.
 bool team64_options(const sso_options* o) {
   return o->precision == SSO_FP64 &&
@@ -1510,7 +1520,8 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
   std::vector<Team64Bin> bins64;
   TeamSpace& space = team_space(B->models[0]->device);
   const int sharers = std::max(1, TeamRuns::count(space));
-  if (o->precision == SSO_FP32_IR && !B->profiling) {
+  if (o->precision == SSO_FP32_IR && !B->profiling &&
+      (!(o->timeout_ms > 0.0) || cluster_pays(o->iters_per_launch, o->precond))) {
     sso_status st = plan_bins(B->n_sys, active, o->precond, sharers, true,
                               [B](int s) { return B->models[s]; }, B->h_list, bins, &cluster);
     if (st != SSO_OK) return st;
@@ -3302,7 +3313,8 @@ sso_status server_upload_tables(sso_server* S, std::vector<std::vector<TileDesc>
   // results are the same bits, and each takes over the other's state)
   S->bins.clear();
   std::vector<int> pack;
-  if (S->opts.precision == SSO_FP32_IR && !S->running.empty()) {
+  if (S->opts.precision == SSO_FP32_IR && !S->running.empty() &&
+      cluster_pays(kServerRounds * S->opts.iters_per_launch, S->opts.precond)) {
     std::vector<char> active(S->max_sys, 0);
     for (int slot : S->running) active[slot] = 1;
     bool fits = false;

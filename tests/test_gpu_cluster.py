@@ -205,11 +205,11 @@ def test_fp64_batches_launches_and_adjoint(sso, precond):
     assert warm.solve(precision="fp64", precond=precond, rtol=1e-10, warm_start=1)["status"] == 0
 
 
-@pytest.mark.parametrize("steps", [1, 2, 3])
+@pytest.mark.parametrize("steps", [1, 4, 5, 6, 7])
 def test_team_launches_begin_in_every_state(sso, steps):
-    # a team per launch of 1 to 3 steps, over several sweeps to convergence:
+    # a team per launch of a few steps, over several sweeps to convergence:
     # launches begin in the first residual, the iteration, the fold and the
-    # residual after it
+    # residual after it (1 step: two kernels)
     m = meshgen.gridshell(110, seed=5)
     kw = dict(rtol=1e-6, inner_rtol=0.1, max_iter=20000)
     want = _same(sso, [m], **kw)
@@ -225,14 +225,28 @@ def test_team_launches_begin_in_every_state(sso, steps):
 def test_team_launch_that_begins_in_the_fold_at_the_cap(sso):
     # the first launch's 1,024 steps end with the last iteration of the cap
     m = meshgen.shell(90, seed=2)
-    kw = dict(rtol=1e-6, max_iter=1023)
-    st = _same(sso, [m], **kw)
+    st = _same(sso, [m], rtol=1e-6, max_iter=1023)
     assert st[0]["iterations"] == 1023 and st[0]["sweeps"] == 1
-    whole = _run(sso, [m], False, **kw)
-    for steps in (1, 2):
+
+
+@pytest.mark.parametrize("size,precond,steps", [
+    (90, "jacobi", 4), (90, "block_jacobi", 4), (20, "jacobi", 4), (20, "block_jacobi", 5),
+    (20, "two_level", 10), (33, "two_level", 13)])
+def test_launches_that_begin_in_the_fold_and_after_it(sso, size, precond, steps):
+    # teams (90 x 90) and clusters; the residual, a sweep of max_iter iterations,
+    # the fold and the second residual: launch 11 begins in the sweep's last
+    # iteration, in the fold, in the residual after it
+    m = meshgen.shell(size, seed=2)
+    for max_iter in (10 * steps, 10 * steps - 1, 10 * steps - 2):
+        kw = dict(rtol=1e-8, precond=precond, inner_rtol=1e-7, max_iter=max_iter)
+        st = _same(sso, [m], **kw)
+        assert st[0]["iterations"] == max_iter and st[0]["sweeps"] == 1
+        whole = _run(sso, [m], False, **kw)
         cut = _run(sso, [m], False, timeout_ms=1e5, iters_per_launch=steps, **kw)
-        assert cut[0][0]["iterations"] == whole[0][0]["iterations"]
-        assert np.array_equal(cut[1][0]["u"], whole[1][0]["u"])
+        for k in ("status", "iterations", "sweeps", "rel_residual"):
+            assert cut[0][0][k] == whole[0][0][k], k
+        for k in ("u", "C", "dz", "dt", "lam"):
+            assert np.array_equal(cut[1][0][k], whole[1][0][k]), k
 
 
 def test_teams_of_several_threads_and_parts(sso):
@@ -280,3 +294,9 @@ def test_fp64_batches_of_unequal_and_many_systems(sso, precond):
     meshes = [meshgen.gridshell(7 + 2 * k, seed=k) for k in range(12)]
     _same(sso, meshes, g=[g.standard_normal(6 * m["xyz"].shape[0]) * (k % 3 == 0)
                           for k, m in enumerate(meshes)], **kw)
+
+
+@pytest.mark.parametrize("side", [191, 233, 234])
+def test_fp64_largest_teams(sso, side):
+    # 1,217 and 1,810 tiles on CTAs of 9 and 12 tiles; 1,826, which takes two kernels
+    _same(sso, [meshgen.gridshell(side, seed=side)], precision="fp64", rtol=1e-10, max_iter=60)
