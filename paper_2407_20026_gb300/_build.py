@@ -21,7 +21,7 @@ def _nvcc():
 
 def _inputs():
     files = [os.path.join(CSRC, f) for f in SOURCES]
-    files.append(os.path.join(CSRC, "sso_internal.cuh"))
+    files += [os.path.join(CSRC, "sso_internal.cuh"), os.path.join(CSRC, "rounding.h")]
     files.append(os.path.join(HERE, "..", "include", "sso.h"))
     return files
 

@@ -57,6 +57,7 @@
 #include <map>
 #include <mutex>
 
+#include "rounding.h"
 #include "sso_internal.cuh"
 
 namespace sso {
@@ -300,9 +301,11 @@ __device__ __forceinline__ bool f64_positive(double x) {
 // of the sum of magnitudes, which may be 2^10 times the sum), the quotient's
 // own: 0.93 2^-34 together.
 // When a float's rounding (or the comparison) is the same anywhere within
-// 2^-34, it is the two-kernel engine's; else, and where a sum leaves the
-// grid's range, the exact sums are formed (exact_sums), about once in 300
-// iterations.
+// 2^-34 of the quotient, it is the two-kernel engine's; else, and where a sum
+// leaves the grid's range, the exact sums are formed (exact_sums): each of an
+// iteration's two quotients fails the test once in 512 times; with a sweep's
+// first iterations, exact sums are formed once in 50 (a few hundred iterations a
+// sweep) to 100 iterations.
 constexpr int kGrid = 50;
 
 __device__ __forceinline__ long long fix_part(float x, int k, unsigned& bad) {
@@ -463,7 +466,7 @@ __device__ __forceinline__ bool apx_fix(const Fix& f, int k, Apx& out) {
   out = apx_bits((unsigned long long)f.s << lz, 63 - lz - k);
   return true;
 }
-// The float nearest a / b; false where 2^-34 more or less would change it.  A
+// The float nearest a / b; false where 2^-34 of it more or less would change it.  A
 // reciprocal, its product, and one remainder step (to 2^-41); then Ziv's test.
 __device__ __forceinline__ bool apx_quotient(const Apx& a, const Apx& b, float& out) {
   float rb;
@@ -473,12 +476,11 @@ __device__ __forceinline__ bool apx_quotient(const Apx& a, const Apx& b, float& 
   const float q1 = __fmul_rn(r, rb);
   const float f = __fadd_rn(q0, q1);
   const float rest = __fsub_rn(q1, __fsub_rn(f, q0));  // q0 + q1 - f, exactly
-  const float half = f < 1.f ? 0x1p-25f : 0x1p-24f;    // of f's last place
   const unsigned fb = __float_as_uint(f);
   const int e = a.e - b.e;
   out = __uint_as_float(fb + ((unsigned)e << 23));
   return e > -100 && e < 100 && a.e > -900 && b.e > -900 && (fb & 0x7fffffu) != 0u &&
-         half - fabsf(rest) > 0x1p-34f;
+         quotient_certain(f, rest);
 }
 // value <= thr for the sum f on the grid 2^-k; sets *clear where the bounds
 // leave no doubt (the sum's own is 2^-33 of it).
