@@ -1652,7 +1652,7 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
       CK(cudaEventRecord(B->ev, B->stream));
       CK(cudaEventSynchronize(B->ev));
       if (B->h_flag[3] != 0)
-        return fail(SSO_ERR_CUDA, "CG kernel gave up waiting for a bulk copy (device fault?)");
+        return fail(SSO_ERR_CUDA, wait_failure(B->h_flag[3]));
       if (B->h_flag[2] <= 0 || launches > max_launches) break;
       if (o->timeout_ms > 0.0 && std::chrono::duration<double, std::milli>(
                                      std::chrono::steady_clock::now() - t0).count() >
@@ -1693,7 +1693,7 @@ sso_status batch_run(sso_batch* B, const sso_options* o, bool adjoint,
       }
       ++launches;
       if (B->h_flag[3] != 0)
-        return fail(SSO_ERR_CUDA, "CG kernel gave up waiting for a bulk copy (device fault?)");
+        return fail(SSO_ERR_CUDA, wait_failure(B->h_flag[3]));
       if (B->h_flag[2] <= 0) break;
       if (o->timeout_ms > 0.0) {
         const double ms = std::chrono::duration<double, std::milli>(
@@ -3815,7 +3815,7 @@ sso_status sso_server_step(sso_server* S, int32_t* n_running, int32_t* n_waiting
     CK(cudaEventSynchronize(B->ev));
     lap(S->ms_wait);
     if (B->h_flag[3] != 0)
-      return fail(SSO_ERR_CUDA, "CG kernel gave up waiting for a bulk copy (device fault?)");
+      return fail(SSO_ERR_CUDA, wait_failure(B->h_flag[3]));
     std::vector<int> done;
     for (int slot : S->running)
       if (B->h_sc[slot].state == ST_DONE) done.push_back(slot);

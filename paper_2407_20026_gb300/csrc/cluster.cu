@@ -425,7 +425,7 @@ __device__ __noinline__ void team_sync(ClShared& sh, bool data) {
     } while (!__all_sync(0xffffffffu, (int)((now - before) >> 48) == sh.team) && --polls);
     if (polls == 0 && lane == 0) {
       sh.lost = 1;
-      atomicExch(sh.flags + 1, 1);
+      atomicExch(sh.flags + 1, WAIT_TEAM);
     }
     if (data) fence_gpu();
     if (lane < 6) sh.before[set][word] = now;

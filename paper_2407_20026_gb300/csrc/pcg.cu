@@ -707,7 +707,7 @@ __global__ void __launch_bounds__(NT, 3) pcg_b32_kernel(const TileDesc* __restri
       const bool ok = mbar_wait(&full[w][s], (k >> 1) & 1);
       if (__any_sync(0xffffffffu, !ok)) {
         dry = true;
-        if (lane == 0) atomicExch(flags + 1, 1);
+        if (lane == 0) atomicExch(flags + 1, WAIT_COPY);
       }
     }
     const SysDesc& S = *J.S;
@@ -1138,7 +1138,7 @@ __global__ void __launch_bounds__(ST_THREADS, 2) pcg_a_staged_kernel(
       const TileDesc td = td_next;
       if (tile + 1 < end) td_next = tiles[tile + 1];
       if (use > 0 && !mbar_wait(&empty[s], (use - 1) & 1)) {
-        atomicExch(flags + 1, 1);
+        atomicExch(flags + 1, WAIT_COPY);
         break;
       }
       const SysDesc* S = sys + td.sys;
@@ -1248,7 +1248,7 @@ __global__ void __launch_bounds__(ST_THREADS, 2) pcg_a_staged_kernel(
     if (!dry && !mbar_wait(&full[s], use & 1)) {
       dry = true;
       s_abort = 1;
-      atomicExch(flags + 1, 1);
+      atomicExch(flags + 1, WAIT_COPY);
     }
     // a dry warp takes nothing from the stage (it may never have been
     // written): the system and its state come from global memory, as the

@@ -146,6 +146,15 @@ struct SysDesc {
   const int* toff;
 };
 
+// Which of a CG kernel's waits ran out (the second of its flags), as an error.
+constexpr int WAIT_COPY = 1, WAIT_TEAM = 2;
+inline const char* wait_failure(int flag) {
+  return flag == WAIT_TEAM
+             ? "a team of CTAs gave up waiting at its barrier (other work held the device's SMs, "
+               "or a device fault)"
+             : "CG kernel gave up waiting for a bulk copy (device fault?)";
+}
+
 #ifdef __CUDACC__
 // Double-float sums of FP32 products: an unevaluated sum hi + lo of two
 // floats, formed only with error-free transformations (the exact product
