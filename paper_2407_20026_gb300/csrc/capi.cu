@@ -1099,9 +1099,24 @@ constexpr double kClusterFixed = 9500.0, kClusterRound = 5000.0;
 // nodes 8.3 -> 8.3, of 90 x 90 12.2 -> 8.3; 64 x 64 shell 7.1 -> 9.4.  Teams
 // need a tile per CTA.
 constexpr double kTeamFixed = 11500.0;
+// The window of a CTA, nodes beyond its own and those that a numbering by rows
+// adds (two rows of 300 and more): a cluster's z goes to every CTA whose window
+// holds the node, a team's CTA reads its window's z and updates p there with its
+// few warps.  Measured with shuffled numbering, 300 iterations, ms, two kernels,
+// choice without and with these terms: 40 x 40 shell 5.2, 4.1, 4.0; 60 x 60 5.7,
+// 10.8, 5.2; grid shells of 50 x 50 nodes 5.3, 6.1, 4.5, 90 x 90 7.8, 13.5, 5.8,
+// 24 of 70 x 70 22.4, 32.4, 22.3 (two kernels).
+constexpr int kRowWindow = 700;
+constexpr double kClusterWindow = 10.0, kTeamWindow = 500.0;  // clocks a node; over its threads
+// The two kernels' clocks of an iteration of all systems (five, two-level).
+double two32_clocks(double tiles, int precond) {
+  return precond == SSO_TWO_LEVEL ? 55000.0 + 25.0 * tiles : 31000.0 + 17.0 * tiles;
+}
 struct ClusterChoice {
   int size = -1;
   bool m_tm = false, team = false;
+  double clocks = 0.0, waves = 0.0;  // of an iteration; rounds for all n_sys
+  bool wide = false;                 // a window beyond a numbering by rows
 };
 ClusterChoice cluster_choice(const sso_model* M, int n_sys, int precond, bool teams,
                              const ClusterDevice& d) {
@@ -1135,7 +1150,9 @@ ClusterChoice cluster_choice(const sso_model* M, int n_sys, int precond, bool te
     if (stream == SIZE_MAX) return;
     if ((size_t)std::min(slots, n_sys) * C * stream > kClusterL2) return;
     const double rounds = (double)sh.own_tiles / warps;
-    const double t = (team ? kTeamFixed : kClusterFixed) + kClusterRound * rounds + stream / 64.0;
+    const double beyond = std::max(0, sh.window - TILE * sh.own_tiles - kRowWindow);
+    const double t = (team ? kTeamFixed : kClusterFixed) + kClusterRound * rounds + stream / 64.0 +
+                     beyond * (team ? kTeamWindow / (32 * warps) : kClusterWindow);
     const double waves = n_sys <= slots ? 1.0
                          : team         ? (double)((n_sys + slots - 1) / slots)
                                         : (double)n_sys / slots;
@@ -1144,6 +1161,9 @@ ClusterChoice cluster_choice(const sso_model* M, int n_sys, int precond, bool te
       best.size = k;
       best.m_tm = m_tm;
       best.team = team;
+      best.clocks = t;
+      best.waves = std::max(1.0, waves);
+      best.wide = beyond > 0.0;
     }
   };
   for (int k = 0; k < CL_SIZES; ++k) consider(false, k);
@@ -1153,7 +1173,8 @@ ClusterChoice cluster_choice(const sso_model* M, int n_sys, int precond, bool te
 }
 
 // Sorts the active systems into launches by cluster size; *fits is false when
-// a system does not fit the engine (the batch then runs the two-kernel engine).
+// a system does not fit the engine, or has a wide window and the estimate of the
+// two-kernel engine is better (the batch then runs that).
 // sharers: batches of about as many systems on the device at the same time;
 // teams: cooperative launches may be used.
 template <class GetModel>
@@ -1168,11 +1189,20 @@ sso_status plan_bins(int n_sys, const std::vector<char>& active, int precond, in
   int n_act = 0;
   for (int s = 0; s < n_sys; ++s) n_act += active[s] != 0;
   std::vector<ClusterChoice> choice(n_sys);
+  double longest = 0.0, all = 0.0, tiles = 0.0;
+  bool wide = false;
   for (int s = 0; s < n_sys; ++s) {
     if (!active[s]) continue;
-    choice[s] = cluster_choice(model(s), n_act * sharers, precond, teams, *dev);
-    if (choice[s].size < 0) return SSO_OK;
+    const ClusterChoice& c = choice[s] =
+        cluster_choice(model(s), n_act * sharers, precond, teams, *dev);
+    if (c.size < 0) return SSO_OK;
+    longest = std::max(longest, c.clocks);
+    all += c.clocks * c.waves / n_act;
+    tiles += model(s)->n_tiles;
+    wide = wide || c.wide;
   }
+  // (with windows of rows, two kernels were faster at no size and count)
+  if (wide && std::max(longest, all) > two32_clocks(sharers * tiles, precond)) return SSO_OK;
   auto collect = [&](bool team, int k, bool m_tm) {
     ClusterBin b{(int)list.size(), 0, team ? cl_team_of(k) : cl_size_of(k), 0, 0, m_tm, team};
     for (int s = 0; s < n_sys; ++s) {

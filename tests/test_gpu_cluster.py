@@ -300,3 +300,67 @@ def test_fp64_batches_of_unequal_and_many_systems(sso, precond):
 def test_fp64_largest_teams(sso, side):
     # 1,217 and 1,810 tiles on CTAs of 9 and 12 tiles; 1,826, which takes two kernels
     _same(sso, [meshgen.gridshell(side, seed=side)], precision="fp64", rtol=1e-10, max_iter=60)
+
+
+def test_teams_beside_a_server(sso):
+    # a server's clusters and set-up kernels between the teams of two batches
+    import threading
+    from paper_2407_20026_gb300.serve import Server
+    opts = sso.options(rtol=1e-4)
+    meshes = [meshgen.gridshell(side, seed=side) for side in (60, 30, 90, 45, 20, 100)] * 2
+    team = [meshgen.shell(90, seed=3), meshgen.gridshell(110, seed=4)]
+    want = _run(sso, team, True, rtol=1e-6, max_iter=900)
+    kw64 = dict(precision="fp64", rtol=1e-10, max_iter=400)
+    small = [meshgen.gridshell(9 + 8 * k, seed=k) for k in range(6)]
+    want64 = _run(sso, small, True, **kw64)
+    got = {}
+
+    def solve(key, ms, kw):
+        got[key] = [_run(sso, ms, False, **kw) for _ in range(3)]
+    threads = [threading.Thread(target=solve, args=a) for a in
+               (("team", team, dict(rtol=1e-6, max_iter=900)), ("fp64", small, kw64))]
+    srv = Server(opts, max_systems=6)
+    tickets = [srv.submit(m) for m in meshes]
+    for t in threads:
+        t.start()
+    while any(srv.step()):
+        pass
+    for t in threads:
+        t.join()
+    for key, ref in (("team", want), ("fp64", want64)):
+        for stats, results in got[key]:
+            for a, b, x, y in zip(stats, ref[0], results, ref[1]):
+                assert (a["status"], a["iterations"]) == (b["status"], b["iterations"])
+                assert np.array_equal(x["u"], y["u"]) and np.array_equal(x["dz"], y["dz"])
+    for m, t in zip(meshes, tickets):
+        mdl = sso.Model(m)
+        mdl.solve(opts)
+        res = srv.poll(t)
+        assert res["stats"]["status"] == 0 and np.array_equal(res["u"], mdl.result()["u"])
+    srv.close()
+
+
+def _shuffled(m, seed):
+    n = m["xyz"].shape[0]
+    perm = np.random.default_rng(seed).permutation(n)
+    inv = np.argsort(perm)
+    m = dict(m)
+    for k in ("beam_conn", "quad_conn"):
+        if len(m[k]):
+            m[k] = inv[m[k]].astype(np.int32)
+    for k in ("xyz", "fixed", "nodal_load"):
+        m[k] = m[k][perm]
+    return m
+
+
+@pytest.mark.parametrize("side,count", [(50, 1), (75, 1), (90, 1), (70, 24)])
+def test_wide_windows(sso, side, count):
+    # shuffled numbering: windows as wide as the system, on clusters, teams and,
+    # where it is faster (24 systems), two kernels an iteration
+    meshes = [_shuffled(meshgen.gridshell(side, seed=k), k) for k in range(count)]
+    kw = dict(rtol=1e-10, max_iter=120)
+    _same(sso, meshes, **kw)
+    before = sso.kernel_launches()
+    sso.Batch([sso.Model(m) for m in meshes]).solve(sso.options(**kw), raise_on_error=False)
+    two_kernels = sso.kernel_launches() - before >= 2 * 120
+    assert two_kernels == (count == 24)
