@@ -11,13 +11,14 @@ FP64 residual of rtol, compliance, and the adjoint dC/dz, dC/dt (Eqs. 5-6).
 
 Prints one JSON line (rank 0).  `value` is designs/s with the designs already
 resident in HBM; `e2e` is the same through the C-ABI from host buffers
-(design upload and result download inside the timed region).  `roofline`
-reports the dominant kernel (CG kernel A: the FP32 BSR SpMV, or the FP64
-residual SpMV in refinement passes), timed live with CUDA events on the
-library's stream in one more, untimed step: a profiled step runs the engine
-of two kernels an iteration, which large systems take; the timed steps run one
-thread-block cluster per design with K on chip and in L2.  `--impl reference` times the FP64 CPU oracle on the same
-workload instead.
+(design upload and result download inside the timed region).
+`roofline_engine` reports the engine of the timed steps, one thread-block
+cluster per design with K on chip and in L2.  `roofline` and `roofline_b` report
+the kernels of the engine of two kernels an iteration, which systems beyond the
+clusters take (kernel A: the FP32 BSR SpMV, or the FP64 residual SpMV in
+refinement passes), timed live with CUDA events on the library's stream in one
+more, untimed step that runs it.  `--impl reference` times the FP64 CPU oracle on
+the same workload instead.
 """
 import argparse
 import hashlib
@@ -36,6 +37,7 @@ sys.path.insert(0, ROOT)
 import meshgen  # noqa: E402
 
 METRIC = "design evals/sec (solve + adjoint grad) at <=1e-6 rel err vs FP64"
+L2_GBS = 20000.0  # L2 reads, 64 B a clock and SM (probed: 19 to 21 TB/s)
 L2_FLUSH_BYTES = 256 << 20
 
 
@@ -957,8 +959,8 @@ def main():
     clocks.start()
     launches0 = sso.kernel_launches()
     step_ms = []
+    cg_ms = []
     iters_total = 0
-    sweeps_total = 0
     for k in range(a.steps):
         flush.fill_(float(k))  # evict L2 between steps
         e0 = torch.cuda.Event(enable_timing=True)
@@ -972,7 +974,7 @@ def main():
         if bad:
             raise RuntimeError("solve failed: %s" % bad[:3])
         iters_total += sum(s["iterations"] for s in stats)
-        sweeps_total += sum(s["sweeps"] for s in stats)
+        cg_ms.append(max(s["ms"] for s in stats))
     torch.cuda.synchronize()
     launches = sso.kernel_launches() - launches0
     clk = clocks.stop()
@@ -1000,8 +1002,8 @@ def main():
     bytes_pcg = nblk * (36 * wsz + 4) + (n_nodes + 1) * 4 + 4 * (6 * n_nodes * wsz)
     bytes_resid = nblk * (36 * 8 + 4) + (n_nodes + 1) * 4 + 3 * (6 * n_nodes * 8)
     alg_bytes = p_iters * bytes_pcg + p_sweeps * bytes_resid
-    step_bytes = (iters_total * (bytes_pcg + 264 * n_nodes) + sweeps_total * bytes_resid)
-    step_gbs = step_bytes / (total_ms / 1000.0) / 1e9  # this GPU
+    cg_bytes = iters_total * bytes_pcg  # of the timed steps
+    cg_gbs = cg_bytes / (sum(cg_ms) / 1000.0) / 1e9
     achieved = alg_bytes / (ms_a / 1000.0) / 1e9 if ms_a > 0 else None
     a_launches = timed_pairs
     traffic = kernel_traffic("pcg.cu", "pcg_a_%s" % ("f32" if fp32 else "f64"))
@@ -1153,16 +1155,16 @@ def main():
                 "kernel_times_from": "profiled step: events around every launch of the engine "
                                      "of two kernels an iteration, the batch run whole (the "
                                      "timed steps run clusters, which stream no K from HBM)",
-                # the timed steps as a whole: the algorithmic bytes of both CG
-                # kernels over the steps' elapsed time (everything else counted
-                # as time), against the same peak; above 1 where K is read from
-                # the chip and L2 instead
-                "step_hbm": {
-                    "achieved": step_gbs, "frac": step_gbs / peak_gbs,
-                    "bytes": step_bytes, "note": "kernel A (SpMV, FP64 residual passes) and "
-                                                 "kernel B (264 B per node) per CG iteration; not "
-                                                 "HBM traffic: the timed steps read K on "
-                                                 "chip and from L2"},
+            },
+            # the engine of the timed steps: kernel A's algorithmic bytes per CG
+            # iteration over the solves' CG time, against what L2 delivers
+            # (beside it registers, tensor and shared memory hold part of K)
+            "roofline_engine": {
+                "bound": "l2, latency", "kernel": "clusters or teams of CTAs (cluster.cu)",
+                "cg_ms_per_step": sum(cg_ms) / a.steps,
+                "us_per_system_iteration": 1e3 * sum(cg_ms) / iters_total,
+                "alg_bytes": cg_bytes, "achieved": cg_gbs, "peak": L2_GBS, "unit": "GB/s",
+                "frac": cg_gbs / L2_GBS, "peak_kind": "L2 reads of a 112 MB set, probed once"
             },
             # elapsed per phase of the profiled step; each set-up stage is
             # one launch for the whole batch
