@@ -286,17 +286,18 @@ sso_status sso_model_get_load(sso_model* model, double* f);
  * Batches: several models (any mix of sizes and topologies, all on the same
  * device) solved together.  Each system runs on a thread-block cluster, or on a
  * team of CTAs of a cooperative launch (large systems, FP64); where a system of
- * the batch fits neither, every CG iteration is one pass of two kernels over
- * all systems that are still iterating.  Each system keeps its own scalars,
- * refinement state and convergence test, and its reductions follow a fixed
- * tiling of its own rows, so its result depends neither on which other systems
- * share the batch nor on which of these runs it.  Solves with teams of several
- * batches of a process take turns.  The batch runs on the stream of models[0].  A batch of 32
- * or more models runs its CG as 2 to 4 parts at once (about 18,000 tiles of 30
- * nodes per part), on the streams of their first models and on as many host
- * threads (the first part on the calling thread); each part's launches overlap
- * the others' tails.  The results are the same bits as without
- * the split (sso_batch_set_parts changes the count).
+ * the batch fits neither, or this should be faster, every CG iteration is one
+ * pass of two kernels over all systems that are still iterating.  Each system
+ * keeps its own scalars, refinement state and convergence test, and its
+ * reductions follow a fixed tiling of its own rows, so its result depends
+ * neither on which other systems share the batch nor on which of these runs it.
+ * Solves with teams of several host threads share a device's SMs, in order of
+ * arrival.  The batch runs on the stream of models[0].  A batch of 32 or more
+ * models runs its CG as 2 to 4 parts at once (about 18,000 tiles of 30 nodes per
+ * part; not FP64 on teams), on the streams of their first models and on as many
+ * host threads (the first part on the calling thread); each part's launches
+ * overlap the others' tails.  The results are the same bits as without the split
+ * (sso_batch_set_parts changes the count).
  */
 sso_status sso_batch_create(sso_model* const* models, int32_t n_models, sso_batch** out);
 

@@ -1595,8 +1595,10 @@ __global__ void __launch_bounds__(KREG ? CL_REG_THREADS : CL_MAX_THREADS, 1) clu
 // six warps on each: a lane per row (five nodes a warp) for the products and
 // the updates, a lane per node for the dot products' trees.
 // Measured, us an iteration, two kernels -> here: 41 x 41 grid shell (10,086 DOF)
-// 26.8 -> 11.6, 100 x 100 39 -> 22.8, 24 x 24 shell 26 -> 12.5; with two kernels
-// under per-launch timing: 64 grid shells of 41 x 41 172 -> 123.
+// 26.8 -> 11.6, 100 x 100 39 -> 22.2, 24 x 24 shell 26 -> 12.5, 64 grid shells of
+// 41 x 41 134 -> 112.  Teams of any sizes share a launch: list holds its systems,
+// then their first CTAs (a launch per size: 32 grid shells of sides 8 to 60 185
+// ms; 40 together, 71 with two kernels).
 template <bool JAC>
 __global__ void __launch_bounds__(TEAM64_THREADS, 1) team64_kernel(
     const SysDesc* __restrict__ sys, const int* __restrict__ list, int* __restrict__ flags,
